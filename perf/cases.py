@@ -225,3 +225,73 @@ def tolerance(case):
     if case["op"] == "dense":
         return {"rel": 8e-3, "max": 0.1}
     return {"rel": 8e-3, "max": 0.9, "differ": 1e-3}
+
+
+def _softmax_rows(q, k, v, logits_more, v_more, allowed, block):
+    """Rows of softmax([q k^T, logits_more]) [v; v_more] where only the key blocks in ``allowed`` [blocks] x rows take part;
+    a row without any key is zero."""
+    x = q @ k.T
+    x.masked_fill_(~allowed.repeat_interleave(block, dim=1)[:, :k.shape[0]], -math.inf)
+    if logits_more is not None:
+        x, v = torch.cat([x, logits_more], dim=1), torch.cat([v, v_more])
+    top = x.amax(dim=1, keepdim=True).clamp_(min=-1e300)
+    x.sub_(top).exp_()
+    return (x @ v) / x.sum(dim=1, keepdim=True).clamp_(min=1e-300)
+
+
+def exact(case, seed):
+    """What ``run`` returns, from the definitions (Eqs. 3-5 and 9-10) in 64 bits.  Counts, bits and orders have no such value: a
+    score within fp32 rounding of its threshold, or of another score, may fall on either side of it."""
+    c = case
+    n, d = _tokens(c), c["d"]
+    if c["op"] != "calibrate" and 4.0 * c["batch"] * c["heads"] * n * n * d > _MOST_FLOPS:
+        return None
+    q, k, v = (x.flatten(0, 1) for x in _inputs(c, seed))
+    block = (64 if d == 64 else 128) if c["op"] == "dense" else c["block"]
+    nb, scale = -(-n // block), 1.0 / math.sqrt(d)
+    sizes = torch.full((nb, 1), float(block), dtype=torch.float64, device="cuda")
+    sizes[-1] = n - (nb - 1) * block
+
+    def pooled(x):
+        return torch.nn.functional.pad(x, (0, 0, 0, nb * block - n)).view(nb, block, d).sum(dim=1) / sizes
+
+    forced = torch.zeros(nb, dtype=torch.bool, device="cuda")
+    if c["forced"]:
+        forced[(n - c["text"]) // block:] = True
+    out = torch.empty(q.shape, dtype=torch.float64, device="cuda") if c["op"] != "calibrate" else None
+    mus, sigmas, taus = [], [], []
+    for h in range(q.shape[0]):
+        qh, kh, vh = q[h].double() * scale, k[h].double(), v[h].double()
+        qb, kc, vc = pooled(qh), pooled(kh), pooled(vh)
+        s = qb @ kc.T
+        mu = s.mean(dim=1)
+        if c["diagonal"]:
+            sigma = (qb.square() @ kc.var(dim=0, correction=0)).sqrt()
+        else:
+            sigma = s.var(dim=1, correction=0).sqrt()
+        tau = mu + c["beta"] * sigma
+        if c["op"] == "topk":
+            keep = max(1, round(c["density"] * nb))
+            ranked = s.sort(dim=1, descending=True).values
+            tau = (ranked[:, keep - 1] + ranked[:, keep]) / 2 if keep < nb else torch.full_like(mu, -math.inf)
+        mus.append(mu), sigmas.append(sigma), taus.append(tau)
+        if out is None:
+            continue
+        chosen = torch.ones_like(s, dtype=torch.bool) if c["op"] == "dense" else (s > tau[:, None]) | forced
+        step = max(1, (1 << 28) // (n * block))                  # query blocks at a time
+        for i in range(0, nb, step):
+            rows = slice(i * block, min(n, (i + step) * block))
+            each = chosen[i:i + step].repeat_interleave(block, dim=0)[:rows.stop - rows.start]
+            more = None
+            if c["op"] != "dense" and c["mode"] == "sol":
+                more = (qh[rows] @ kc.T + sizes.log().T).masked_fill_(each, -math.inf)
+            out[h, rows] = _softmax_rows(qh[rows], kh, vh, more, vc, each, block)
+    if out is not None:
+        out = out.view(c["batch"], c["heads"], n, d)
+        out = out.transpose(1, 2).contiguous() if c["tokens_first"] else out
+    mu, sigma, tau = (torch.stack(x).view(c["batch"], c["heads"], nb) for x in (mus, sigmas, taus))
+    if c["op"] == "calibrate":
+        return mu, sigma, tau, None
+    if c["op"] == "topk":
+        return out, None, None, tau
+    return (out, None, None) if c["prepass"] else (out, None)
