@@ -1,8 +1,8 @@
 // Sol-Attn fused forward (Algorithm 1) for sm_100a: TMA + tcgen05.mma + TMEM.
 //
-// Persistent kernel, one CTA of 384 threads per SM, compiled for d in {64, 128} and
-// block_q = block_k in {64, 128}.  A CTA owns one query block at a time and is split into warp
-// roles that talk through mbarriers:
+// Persistent kernel for 128-token blocks, one CTA of 384 threads per SM, compiled for d in {64, 128}
+// (fwd_sm100_b64.cu is the one for 64-token blocks).  A CTA owns one query block at a time and is split
+// into warp roles that talk through mbarriers:
 //
 //   router   (warp 8)  pulls (head, query block) work items from a global counter and walks the
 //                      pooled keys in chunks of `block` blocks.  For every block it evaluates the
@@ -26,10 +26,6 @@
 //                      padded columns.  O_h is rescaled lazily, only when the running maximum
 //                      grows by more than 2^8.
 //
-// The query tile of the MMAs always has 128 rows (the M of a one-CTA tcgen05.mma at full rate);
-// with 64-token blocks its upper 64 rows belong to the next query block, take part in the
-// arithmetic and are never stored.
-//
 // TMEM (512 columns): S0 [0, block)  S1 [block, 2 block)  O0 [256, 256 + d)  O1 [256 + d, 256 + 2 d);
 // P_h (bf16) of a tile overwrites the start of group h's half of that tile's S buffer.
 //
@@ -37,25 +33,18 @@
 // workspace status word, all roles drain, TMEM is released and the kernel returns.
 #include <type_traits>
 
-#include "common.cuh"
-#include "ptx_sm100.cuh"
-#include "tmap.cuh"
+#include "fwd_sm100_common.cuh"
 
 namespace sol {
+namespace fwd {
 namespace {
 
-using namespace ptx;
-
-constexpr int kRowsQ = 128;                      // rows of the query tile fed to the tensor core
-constexpr int kThreads = 384;
 constexpr int kKStages = 2;                      // ring of K tiles
 constexpr int kVStages = 2;                      // ring of V tiles (its own ring: the score GEMMs run ahead of P V)
 constexpr int kGroup = 32;                       // pooled keys scored per router step (one per lane)
 constexpr int kRecords = 4;                      // ring of routing records
-constexpr int kWarpRouter = 8, kWarpProducer = 9, kWarpQK = 10;   // warp 11 issues P V
-constexpr int kTmemCols = 512;
+constexpr int kWarpQK = 10;                      // warp 11 issues P V
 constexpr int kTmemS = 0, kTmemO = 256;
-constexpr float kRescaleThreshold = 8.0f;        // log2 units
 
 // Compile-time shape of one kernel instance.
 template <int D, int BLK>
@@ -69,7 +58,7 @@ struct Cfg {
   static constexpr int kQBoxBytes = kRowsQ * 128;  // one box of the query tile (64 channels x 128 rows)
   static constexpr int kBoxBytes = BLK * 128;      // one box of a K-like / V-like tile
   static_assert(D == 64 || D == 128, "head dimension");
-  static_assert(BLK == 64 || BLK == 128, "block size");
+  static_assert(BLK == kRowsQ, "a query block fills the query tile");
 };
 
 // The router turns every chunk of `block` key blocks into a record: a flat list of tile descriptors
@@ -109,32 +98,8 @@ struct Shared {
   int abort_flag;
 };
 
-struct Params {
-  const float* qbar;            // [BH][Nq][d]
-  const float* kc;              // [BH][Nk][d]
-  const float* tau;             // [BH][Nq]
-  __nv_bfloat16* out;
-  int32_t* counts;
-  uint32_t* mask_out;
-  int32_t* status;              // workspace status words
-  int N, Nq, Nk, total_work, mode;
-  float scale;
-  const uint8_t* forced;        // [Nk] or null: key blocks always routed to the exact branch
-  Strides st;                   // layout of q, k, v, out
-  int rows_inner;               // coordinate order of the q/k/v tensor maps: (c, row, h, b) or (c, h, row, b)
-  long long wait_limit;         // SM clocks after which a bounded wait gives up
-  int withhold_tile;            // test hook: >= 0: the P V role leaves out the completion signal of this tile
-  int out_aligned32;            // every output row piece starts on a 32-byte boundary (32-byte stores are legal)
-};
-
-template <class S>
-__device__ __forceinline__ void flag_abort(S& sm, const Params& p, int where) {
-  sm.abort_flag = 1;
-  atomicExch(p.status + kStatusDevice, (int)SOL_ERR_DEVICE_TIMEOUT);
-  atomicCAS(p.status + kStatusDetail, 0, where);     // keep the first place that gave up
-}
-
 }  // namespace
+}  // namespace fwd
 }  // namespace sol
 
 // Every role has `sm` and `wait_limit` in scope; WAIT is a bounded wait on one of its barriers.
@@ -159,6 +124,7 @@ __device__ __forceinline__ void flag_abort(S& sm, const Params& p, int where) {
 #endif
 
 namespace sol {
+namespace fwd {
 namespace {
 
 // ------------------------------------------------------------------------------------------------
@@ -485,13 +451,6 @@ __device__ void producer_role(Shared<C>& sm, const Params& p, unsigned char* sQ,
 // bookkeeping of one kind of MMA delays the other; the tensor pipe arbitrates between them and all
 // ordering is carried by the mbarriers.
 //
-// Shared-memory descriptors: the upper word is constant (stride 1024 B between 8-row groups,
-// descriptor version, 128-byte swizzle); the lower word is (address >> 4) | (leading offset >> 4) << 16.
-__device__ __forceinline__ uint64_t desc_from_lo(uint32_t lo) {
-  constexpr uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);
-  return ((uint64_t)hi << 32) | lo;
-}
-
 // Abort path of an MMA-issuing role: TMEM must not be released while MMAs are still writing to it, so
 // the role asks for a completion signal behind everything it has issued and waits for it (bounded).
 template <class C>
@@ -626,12 +585,6 @@ __device__ void mma_pv_role(Shared<C>& sm, const Params& p, unsigned char* sKV, 
 // ------------------------------------------------------------------------------------------------
 // softmax + correction + epilogue: two warpgroups of 128 threads; thread = query row, warpgroup h
 // owns key columns [kHalf h, kHalf (h+1)) of every tile.
-template <int N>
-__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t* r) {   // N columns, N a multiple of 32
-#pragma unroll
-  for (int c = 0; c < N; c += 32) tmem_ld_32x32b_x32(taddr + c, *reinterpret_cast<uint32_t(*)[32]>(r + c));
-}
-
 template <class C>
 __device__ void softmax_role(Shared<C>& sm, const Params& p, uint32_t tmem, int h, int warp_in_group, int lane) {
   constexpr int kD = C::kD, kBlk = C::kBlk, kHalf = C::kHalf;
@@ -924,60 +877,27 @@ long long g_wait_limit = kWaitCycles;
 int g_withhold_tile = -1;
 
 template <class C>
-cudaError_t launch_instance(const Problem& p, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
-                            __nv_bfloat16* out, const WsPtrs& ws, const float* tau, int32_t* counts, uint32_t* mask_out,
-                            cudaStream_t stream, int* n_launches) {
-  CUtensorMap tq, tk, tv, tkc, tvm;
-  bool rows_inner = true, pooled_inner = true;
-  auto user_map = [&](CUtensorMap* m, const void* base, int box_rows) {
-    return make_tmap_bf16_4d(m, base, p.B, p.H, p.N, C::kD, box_rows, p.st.row, p.st.head, p.st.batch, &rows_inner);
-  };
-  auto pooled_map = [&](CUtensorMap* m, const void* base) {      // dense [B][H][Nk][d]
-    return make_tmap_bf16_4d(m, base, p.B, p.H, p.Nk, C::kD, C::kBlk, C::kD, (long long)p.Nk * C::kD,
-                             (long long)p.H * p.Nk * C::kD, &pooled_inner);
-  };
-  if (!user_map(&tq, q, kRowsQ) || !user_map(&tk, k, C::kBlk) || !user_map(&tv, v, C::kBlk) ||
-      !pooled_map(&tkc, ws.kcb) || !pooled_map(&tvm, ws.vmb) || !pooled_inner)
-    return cudaErrorInvalidValue;
-  Params prm{};
-  prm.qbar = ws.qbar; prm.kc = ws.kc; prm.tau = tau; prm.out = out; prm.counts = counts; prm.mask_out = mask_out;
-  prm.status = ws.status; prm.N = p.N; prm.Nq = p.Nq; prm.Nk = p.Nk; prm.total_work = p.BH * p.Nq;
-  prm.mode = p.mode; prm.scale = p.scale; prm.forced = p.forced;
-  prm.st = p.st; prm.rows_inner = rows_inner ? 1 : 0;
-  prm.wait_limit = g_wait_limit; prm.withhold_tile = g_withhold_tile;
-  prm.out_aligned32 = (reinterpret_cast<uintptr_t>(out) % 32 == 0 && (p.st.row * 2) % 32 == 0 && (p.st.head * 2) % 32 == 0 &&
-                       (p.st.batch * 2) % 32 == 0) ? 1 : 0;
-
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
+cudaError_t launch_instance(const Problem& p, const Maps& m, const Params& prm, int grid, cudaStream_t stream) {
   const size_t smem = 1024 + C::kQBytes + (kKStages + kVStages) * C::kTileBytes + sizeof(Shared<C>);
-  const int grid = prm.total_work < sms ? prm.total_work : sms;
   // the pre-pass variant is a kernel of its own, so that the in-kernel router's code is what it is without it
-  if (p.routing == SOL_ROUTING_PREPASS && p.mode != SOL_MODE_DENSE) {
-    e = cudaFuncSetAttribute(fwd_sm100_kernel<C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    fwd_sm100_kernel<C, true><<<grid, kThreads, smem, stream>>>(tq, tk, tv, tkc, tvm, prm);
-  } else {
-    e = cudaFuncSetAttribute(fwd_sm100_kernel<C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    fwd_sm100_kernel<C, false><<<grid, kThreads, smem, stream>>>(tq, tk, tv, tkc, tvm, prm);
-  }
-  if (n_launches) *n_launches += 1;
+  auto kernel = p.routing == SOL_ROUTING_PREPASS && p.mode != SOL_MODE_DENSE ? fwd_sm100_kernel<C, true>
+                                                                            : fwd_sm100_kernel<C, false>;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kernel<<<grid, kThreads, smem, stream>>>(m.q, m.k, m.v, m.kc, m.vm, prm);
   return cudaGetLastError();
 }
 
 }  // namespace
+}  // namespace fwd
 
 bool fwd_sm100_supports(const Problem& p) {
   return (p.d == 64 || p.d == 128) && p.block_q == p.block_k && (p.block_k == 64 || p.block_k == 128);
 }
 
 void fwd_sm100_set_wait(long long wait_cycles, int withhold_tile) {
-  g_wait_limit = wait_cycles > 0 ? wait_cycles : kWaitCycles;
-  g_withhold_tile = withhold_tile;
+  fwd::g_wait_limit = wait_cycles > 0 ? wait_cycles : ptx::kWaitCycles;
+  fwd::g_withhold_tile = withhold_tile;
 }
 
 cudaError_t launch_fwd_sm100(const Problem& p, const __nv_bfloat16* q, const __nv_bfloat16* k,
@@ -985,13 +905,23 @@ cudaError_t launch_fwd_sm100(const Problem& p, const __nv_bfloat16* q, const __n
                              int32_t* counts, uint32_t* mask_out, cudaStream_t stream,
                              int* n_launches) {
   if (!fwd_sm100_supports(p)) return cudaErrorInvalidValue;
-  if (p.d == 128 && p.block_k == 128)
-    return launch_instance<Cfg<128, 128>>(p, q, k, v, out, ws, tau, counts, mask_out, stream, n_launches);
-  if (p.d == 64 && p.block_k == 64)
-    return launch_instance<Cfg<64, 64>>(p, q, k, v, out, ws, tau, counts, mask_out, stream, n_launches);
-  if (p.d == 128)
-    return launch_instance<Cfg<128, 64>>(p, q, k, v, out, ws, tau, counts, mask_out, stream, n_launches);
-  return launch_instance<Cfg<64, 128>>(p, q, k, v, out, ws, tau, counts, mask_out, stream, n_launches);
+  if (p.block_k == 64)
+    return fwd::launch_b64(p, q, k, v, out, ws, tau, counts, mask_out, fwd::g_wait_limit, fwd::g_withhold_tile, stream,
+                           n_launches);
+  fwd::Maps m;
+  fwd::Params prm;
+  if (!fwd::prepare(p, q, k, v, out, ws, tau, counts, mask_out, &m, &prm)) return cudaErrorInvalidValue;
+  prm.total_work = p.BH * p.Nq;
+  prm.wait_limit = fwd::g_wait_limit;
+  prm.withhold_tile = fwd::g_withhold_tile;
+  int sms = 0;
+  cudaError_t e = fwd::sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  const int grid = prm.total_work < sms ? prm.total_work : sms;
+  e = p.d == 128 ? fwd::launch_instance<fwd::Cfg<128, 128>>(p, m, prm, grid, stream)
+                 : fwd::launch_instance<fwd::Cfg<64, 128>>(p, m, prm, grid, stream);
+  if (n_launches) *n_launches += 1;
+  return e;
 }
 
 }  // namespace sol
