@@ -95,13 +95,13 @@ sol::Problem make_problem(int B, int H, int N, int d, int block_q, int block_k, 
   return p;
 }
 
-sol_status_t run_pool(const sol::Problem& p, const void* q, const void* k, const void* v, void* ws_base,
+sol_status_t run_pool(const sol::Problem& p, const void* q, const void* k, const void* v, void* ws_base, int zero_from,
                       cudaStream_t stream) {
   const sol::WsLayout lay = sol::make_layout(p.BH, p.Nq, p.Nk, p.d);
   const sol::WsPtrs ws = sol::make_ptrs(ws_base, lay);
   int n = 0;
   cudaError_t e = sol::launch_pool(p, static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k),
-                                   static_cast<const __nv_bfloat16*>(v), ws, stream, &n);
+                                   static_cast<const __nv_bfloat16*>(v), ws, zero_from, stream, &n);
   if (e == cudaSuccess && q) e = sol::launch_thresholds(p, ws, stream, &n);
   g_launches += n;
   return e == cudaSuccess ? SOL_OK : SOL_ERR_CUDA;
@@ -172,7 +172,7 @@ sol_status_t sol_attn_pool(const void* q, const void* k, const void* v, int B, i
   if (g_bound.bytes < sol_attn_workspace_bytes(B, H, N, d, block_q, block_k)) return SOL_ERR_WORKSPACE;
   if ((s = check_arch()) != SOL_OK) return s;
   const sol::Problem p = make_problem(B, H, N, d, block_q, block_k, threshold, 0.f, SOL_MODE_SOL);
-  return run_pool(p, q, k, v, g_bound.ws, static_cast<cudaStream_t>(stream));
+  return run_pool(p, q, k, v, g_bound.ws, sol::kStatusWords, static_cast<cudaStream_t>(stream));
 }
 
 sol_status_t sol_attn_thresholds(int B, int H, int N, int d, int block_q, int block_k, float threshold, float scale,
@@ -245,12 +245,12 @@ static sol_status_t forward_impl(const sol_attn_args* a, bool keep_status) {
   const sol::WsLayout lay = sol::make_layout(p.BH, p.Nq, p.Nk, p.d);
   const sol::WsPtrs ws = sol::make_ptrs(a->workspace, lay);
   const int first_word = keep_status ? sol::kStatusTileCounter : 0;
-  if (cudaMemsetAsync(ws.status + first_word, 0, sizeof(int32_t) * (sol::kStatusWords - first_word), stream) !=
-      cudaSuccess)
-    return SOL_ERR_CUDA;
   if (p.mode != SOL_MODE_DENSE && !a->skip_pool) {
-    s = run_pool(p, a->q, a->k, a->v, a->workspace, stream);
+    s = run_pool(p, a->q, a->k, a->v, a->workspace, first_word, stream);   // zeroes the status words too
     if (s != SOL_OK) return s;
+  } else if (cudaMemsetAsync(ws.status + first_word, 0, sizeof(int32_t) * (sol::kStatusWords - first_word), stream) !=
+             cudaSuccess) {
+    return SOL_ERR_CUDA;
   }
   const float* tau = a->tau_override ? a->tau_override : ws.tau;
   int n = 0;

@@ -15,7 +15,6 @@ constexpr int kStatusWords = 16;      // int32 words at the start of the workspa
 constexpr int kStatusDevice = 0;      // word 0: device status (0 ok, SOL_ERR_DEVICE_TIMEOUT ...)
 constexpr int kStatusDetail = 1;      // word 1: where a bounded wait gave up (debug aid)
 constexpr int kStatusTileCounter = 2; // word 2: persistent-kernel work counter
-constexpr int kCovSlices = 4;         // partial second-moment matrices per (batch, head)
 
 __host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -52,8 +51,8 @@ struct WsLayout {
   size_t vc;      // fp32 [BH][Nk][d]   sum of each value block         (before Eq. 9)
   size_t kcb;     // bf16 [BH][Nk][d]   KC rounded, MMA operand of the approximate branch
   size_t vmb;     // bf16 [BH][Nk][d]   VC / n_j rounded, MMA operand of the approximate branch
-  size_t mk;      // fp32 [BH][d]       first moment of the pooled keys (Eq. 5)
-  size_t covk;    // fp32 [kCovSlices][BH][d][d]  partial centred second moments of the pooled keys (Eq. 5)
+  size_t mk;      // fp32 [BH][d]       diagonal estimator: first moment of the pooled keys
+  size_t vk;      // fp32 [BH][d]       diagonal estimator: channel variances of the pooled keys
   size_t mu, sigma, tau;  // fp32 [BH][Nq] each (Eq. 4)
   size_t total;
 };
@@ -69,7 +68,7 @@ inline WsLayout make_layout(int BH, int Nq, int Nk, int d) {
   w.kcb = take(2 * (size_t)BH * Nk * d);
   w.vmb = take(2 * (size_t)BH * Nk * d);
   w.mk = take(sizeof(float) * (size_t)BH * d);
-  w.covk = take(sizeof(float) * (size_t)kCovSlices * BH * d * d);
+  w.vk = take(sizeof(float) * (size_t)BH * d);
   w.mu = take(sizeof(float) * (size_t)BH * Nq);
   w.sigma = take(sizeof(float) * (size_t)BH * Nq);
   w.tau = take(sizeof(float) * (size_t)BH * Nq);
@@ -82,7 +81,7 @@ struct WsPtrs {
   int32_t* status;
   float *qbar, *kc, *vc;
   __nv_bfloat16 *kcb, *vmb;
-  float *mk, *covk, *mu, *sigma, *tau;
+  float *mk, *vk, *mu, *sigma, *tau;
 };
 
 inline WsPtrs make_ptrs(void* base, const WsLayout& w) {
@@ -95,7 +94,7 @@ inline WsPtrs make_ptrs(void* base, const WsLayout& w) {
   p.kcb = reinterpret_cast<__nv_bfloat16*>(b + w.kcb);
   p.vmb = reinterpret_cast<__nv_bfloat16*>(b + w.vmb);
   p.mk = reinterpret_cast<float*>(b + w.mk);
-  p.covk = reinterpret_cast<float*>(b + w.covk);
+  p.vk = reinterpret_cast<float*>(b + w.vk);
   p.mu = reinterpret_cast<float*>(b + w.mu);
   p.sigma = reinterpret_cast<float*>(b + w.sigma);
   p.tau = reinterpret_cast<float*>(b + w.tau);
@@ -108,9 +107,10 @@ sol_status_t check_device_arch();      // SOL_OK on compute capability 10.x, els
 
 // ---- launchers (each returns the cudaError_t of its launches; all work goes to `stream`) ----
 
-// Pooling pre-pass: Qbar, KC, VC (+ bf16 operand copies).  q may be null.
+// Pooling pre-pass: Qbar, KC, VC (+ bf16 operand copies).  q may be null.  The status words from `zero_from` on
+// are zeroed along the way (kStatusWords: none).
 cudaError_t launch_pool(const Problem& p, const __nv_bfloat16* q, const __nv_bfloat16* k,
-                        const __nv_bfloat16* v, const WsPtrs& ws, cudaStream_t stream, int* n_launches);
+                        const __nv_bfloat16* v, const WsPtrs& ws, int zero_from, cudaStream_t stream, int* n_launches);
 
 // Pooled-key moments (Eq. 5) and per-query-block mu, sigma, tau (Eq. 4).
 cudaError_t launch_thresholds(const Problem& p, const WsPtrs& ws, cudaStream_t stream, int* n_launches);

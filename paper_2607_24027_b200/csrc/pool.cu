@@ -3,6 +3,10 @@
 //
 // The pooling kernel is HBM-bound: it reads q, k and v exactly once with 16-byte loads and
 // writes a few MB of pooled vectors.  The moment / threshold kernels touch only pooled data.
+#include <cooperative_groups.h>
+
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace sol {
@@ -22,10 +26,13 @@ template <int D>
 __global__ void __launch_bounds__(kPoolThreads)
 pool_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
             const __nv_bfloat16* __restrict__ v, WsPtrs ws, Strides st, int N, int block_q, int block_k,
-            int Nq, int Nk, int first_kind) {
+            int Nq, int Nk, int first_kind, int zero_from) {
   constexpr int TPR = D / 8;                    // threads per row
   constexpr int RG = kPoolThreads / TPR;        // row groups
   __shared__ float partial[RG][D];
+
+  // the call's status words, which the fused kernel behind this one counts in
+  if (blockIdx.x == 0 && threadIdx.x >= zero_from && threadIdx.x < kStatusWords) ws.status[threadIdx.x] = 0;
 
   // blockIdx.x enumerates, per (batch, head): Nq query blocks (if q is pooled), Nk key blocks,
   // Nk value blocks.
@@ -99,143 +106,302 @@ pool_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict
   }
 }
 
-// First moment of the pooled keys, m_K = (1/Nk) sum_j KC_j  (Eq. 5).  One CTA per (batch, head):
-// 4 row groups x D channels, combined through shared memory.
-template <int D>
-__global__ void __launch_bounds__(4 * D) key_mean_kernel(WsPtrs ws, int Nk) {
-  __shared__ float part[4][D];
-  const int bh = blockIdx.x, c = threadIdx.x % D, grp = threadIdx.x / D;
-  const float* kc = ws.kc + (size_t)bh * Nk * D;
-  float s0 = 0.f, s1 = 0.f;
-  int j = grp;
-  for (; j + 4 < Nk; j += 8) {
-    s0 += kc[(size_t)j * D + c];
-    s1 += kc[(size_t)(j + 4) * D + c];
-  }
-  if (j < Nk) s0 += kc[(size_t)j * D + c];
-  part[grp][c] = s0 + s1;
-  __syncthreads();
-  if (grp == 0) ws.mk[(size_t)bh * D + c] = ((part[0][c] + part[1][c]) + (part[2][c] + part[3][c])) / (float)Nk;
+// mu, sigma and tau of one query block, from its raw products.
+__device__ __forceinline__ void store_threshold(const WsPtrs& ws, size_t o, float mu, float sigma, float beta) {
+  ws.mu[o] = mu;
+  ws.sigma[o] = sigma;
+  ws.tau[o] = isinf(beta) ? beta : fmaf(beta, sigma, mu);   // +inf: route nothing, -inf: route everything
 }
 
-// Centred second moment of the pooled keys,
-//   C_K = (1/Nk) sum_j (KC_j - m_K)^T (KC_j - m_K)  =  (1/Nk) sum_j KC_j^T KC_j - m_K^T m_K,
-// i.e. the bracket of Eq. (5) with the mu_i^2 term already folded in, which avoids the
-// cancellation of the uncentred form in fp32.  Grid (D/16, BH, key slices); a CTA of 256 threads
-// owns 16 rows of C_K for one slice of the pooled keys, thread (r, cg) owns C_K[r][cg*8 ..
-// cg*8+7]; every slice writes its own partial matrix (covk holds kCovSlices of them per launch,
-// slice-major) and tau_kernel adds them in a fixed order, so the result is bit-stable run to run.
+// Thresholds of a head with few pooled keys (Nk <= kSmallKeys), in one launch.  A CTA takes 16 query blocks
+// of one head, with all pooled keys of the head in shared memory: mean, then centred keys x_j = KC_j - m_K,
+// then the row statistics straight from the centred scores,
+//   mu_i = s Qbar_i . m_K,   sigma_i^2 = s^2 (1/Nk) sum_j (Qbar_i . x_j)^2,
+// which is Eq. (4)'s own definition (and Eq. 5's quadratic form with the sums exchanged).  With kDiag the
+// diagonal estimator: sigma_i^2 = s^2 (Qbar_i o Qbar_i) . v_K, v_K = (1/Nk) sum_j x_j o x_j.
+//
+// These sizes are bound by latency: a launch and a few dependent passes over a few KB.  24 heads of 32 key and
+// 32 query blocks, d = 128: 6.4 us, where the three kernels of the moments (mean, second moment, quadratic
+// form) took 42 us and two more launches.  Its work grows with Nq Nk, that of the second moment with
+// (Nq + Nk) d, so the line lies at Nk = d.
+constexpr int kSmallKeys = 128, kSmallRows = 16;
+
+template <int D, bool kDiag>
+__global__ void __launch_bounds__(256) thresholds_small_kernel(WsPtrs ws, int Nq, int Nk, float scale, float beta) {
+  constexpr int LD = D + 4;                      // rows 4 banks apart: 16-byte reads of eight rows do not collide
+  constexpr int G = 256 / D;                     // threads per channel
+  extern __shared__ float smem_f[];
+  float* ks = smem_f;                            // [Nk][LD]
+  __shared__ float qs[kSmallRows][LD];
+  __shared__ float part[G][D], mean_s[D], var_s[kDiag ? D : 1];
+  const int bh = blockIdx.y, i0 = blockIdx.x * kSmallRows, tid = threadIdx.x;
+  const float* kc = ws.kc + (size_t)bh * Nk * D;
+  const float* qb = ws.qbar + ((size_t)bh * Nq + i0) * D;
+  const int nq = min(kSmallRows, Nq - i0);
+#pragma unroll 4
+  for (int e = tid; e < Nk * (D / 4); e += 256)
+    *reinterpret_cast<float4*>(ks + (e / (D / 4)) * LD + (e % (D / 4)) * 4) = reinterpret_cast<const float4*>(kc)[e];
+  for (int e = tid; e < kSmallRows * (D / 4); e += 256)
+    *reinterpret_cast<float4*>(&qs[e / (D / 4)][(e % (D / 4)) * 4]) =
+        e / (D / 4) < nq ? reinterpret_cast<const float4*>(qb)[e] : make_float4(0.f, 0.f, 0.f, 0.f);
+  __syncthreads();
+  const int c = tid % D, g = tid / D;
+  auto total = [&](float s) {                    // sum over the G threads of a channel, in a fixed order
+    part[g][c] = s;
+    __syncthreads();
+    float r = 0.f;
+#pragma unroll
+    for (int x = 0; x < G; ++x) r += part[x][c];
+    __syncthreads();
+    return r;
+  };
+  float s = 0.f;
+#pragma unroll 8
+  for (int j = g; j < Nk; j += G) s += ks[j * LD + c];
+  const float m = total(s) / (float)Nk;
+  float sq = 0.f;
+#pragma unroll 8
+  for (int j = g; j < Nk; j += G) {
+    const float x = ks[j * LD + c] - m;
+    if constexpr (kDiag) sq = fmaf(x, x, sq);
+    else ks[j * LD + c] = x;
+  }
+  if constexpr (kDiag) {
+    const float v = total(sq) / (float)Nk;
+    if (g == 0) var_s[c] = v;
+  }
+  if (g == 0) mean_s[c] = m;
+  __syncthreads();
+  const int row = tid / 16, tx = tid % 16;
+  float quad = 0.f, dotm = 0.f;
+  if constexpr (!kDiag) {
+    const float4* q4 = reinterpret_cast<const float4*>(qs[row]);
+    for (int j = tx; j < Nk; j += 32) {          // two keys at a time
+      const bool two = j + 16 < Nk;
+      const float4* ka = reinterpret_cast<const float4*>(ks + j * LD);
+      const float4* kb = two ? ka + 16 * (LD / 4) : ka;
+      float2 a0 = make_float2(0.f, 0.f), a1 = a0, b0 = a0, b1 = a0;
+#pragma unroll 8
+      for (int p = 0; p < D / 4; ++p) {
+        const float4 q = q4[p], x = ka[p], y = kb[p];
+        a0 = __ffma2_rn(make_float2(q.x, q.y), make_float2(x.x, x.y), a0);
+        a1 = __ffma2_rn(make_float2(q.z, q.w), make_float2(x.z, x.w), a1);
+        b0 = __ffma2_rn(make_float2(q.x, q.y), make_float2(y.x, y.y), b0);
+        b1 = __ffma2_rn(make_float2(q.z, q.w), make_float2(y.z, y.w), b1);
+      }
+      const float sa = (a0.x + a0.y) + (a1.x + a1.y), sb = (b0.x + b0.y) + (b1.x + b1.y);
+      quad = fmaf(sa, sa, quad);
+      if (two) quad = fmaf(sb, sb, quad);
+    }
+    quad /= (float)Nk;
+  }
+#pragma unroll
+  for (int p = 0; p < D / 16; ++p) {
+    const float q = qs[row][tx + 16 * p];
+    dotm = fmaf(q, mean_s[tx + 16 * p], dotm);
+    if constexpr (kDiag) quad = fmaf(q * q, var_s[tx + 16 * p], quad);
+  }
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) {
+    quad += __shfl_xor_sync(0xffffffffu, quad, o);
+    dotm += __shfl_xor_sync(0xffffffffu, dotm, o);
+  }
+  if (tx == 0 && row < nq)
+    store_threshold(ws, (size_t)bh * Nq + i0 + row, scale * dotm, scale * sqrtf(fmaxf(quad, 0.f)), beta);
+}
+
+// Thresholds of a head with many pooled keys, in one launch: the moments m_K and
+//   C_K = (1/Nk) sum_j (KC_j - m_K)^T (KC_j - m_K)
+// (the bracket of Eq. 5 with the mu_i^2 term already folded in, which avoids the cancellation of the
+// uncentred form in fp32), then per query block mu_i = s Qbar_i . m_K, sigma_i^2 = s^2 Qbar_i C_K Qbar_i^T.
+//
+// A thread-block cluster takes one head.  Each CTA sums its share of the keys, first for the mean, then for a
+// partial C_K in registers (256 threads, 8 x 8 or 4 x 4 each); the partial sums are added through distributed
+// shared memory in rank order (bit-stable run to run), every CTA gathers the whole C_K and forms Y = Qbar C_K for
+// its share of the query blocks.  FMA-bound: 1.5 GFLOP at 40 heads x 591 blocks, d = 128, 92 us, where
+// three kernels (mean on 40 CTAs; C_K with one shared-memory operand per FMA; quadratic form) took 198 us.
+constexpr int kMomentRows = 80;                  // query blocks per step: 5 for each of 16 thread rows
 
 template <int D>
-__global__ void __launch_bounds__(256) key_cov_kernel(WsPtrs ws, int Nk) {
-  constexpr int ROWS = 16;
-  constexpr int CG = 256 / ROWS;                 // column groups per row (16)
-  constexpr int CPT = D / CG;                    // columns per thread (8 or 4)
-  constexpr int JT = 32;                         // pooled keys staged per step
-  __shared__ float xs[JT][D];
-  const int bh = blockIdx.y;
-  const int r = blockIdx.x * ROWS + threadIdx.x / CG;
-  const int c0 = (threadIdx.x % CG) * CPT;
+constexpr size_t moments_smem() {                // C_K, then (in turn) staged keys / a reduced strip / pooled queries
+  constexpr size_t work = sizeof(float) * kMomentRows * (D + 4), strip = sizeof(float) * D * D / 2;
+  return sizeof(float) * D * D + (work > strip ? work : strip);
+}
+
+template <int D>
+__global__ void __launch_bounds__(256, 2) thresholds_moments_kernel(WsPtrs ws, int Nq, int Nk, float scale, float beta) {
+  constexpr int T = D / 16;                      // C_K rows and columns per thread (8 or 4)
+  constexpr int JT = 32;                         // keys staged per step
+  constexpr int G = 256 / D;
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int n_cta = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  extern __shared__ __align__(16) float smem_f[];
+  float* cov = smem_f;                           // [D][D]
+  float* work = smem_f + D * D;
+  __shared__ float part[G][D], sum_s[D], mean_s[D];
+  const int bh = blockIdx.y, tid = threadIdx.x;
+  const int ty = tid / 16, tx = tid % 16;
   const float* kc = ws.kc + (size_t)bh * Nk * D;
-  const float* mk = ws.mk + (size_t)bh * D;
-  const int per_slice = ceil_div(Nk, kCovSlices);
-  const int j_begin = blockIdx.z * per_slice, j_end = min(Nk, j_begin + per_slice);
-  float acc[CPT];
+  const int per_k = ceil_div(Nk, n_cta);
+  const int j_begin = min(Nk, rank * per_k), j_end = min(Nk, j_begin + per_k);
+
+  // ---- m_K
+  {
+    const int c = tid % D, g = tid / D;
+    float s = 0.f;
+#pragma unroll 8
+    for (int j = j_begin + g; j < j_end; j += G) s += kc[(size_t)j * D + c];
+    part[g][c] = s;
+    __syncthreads();
+    if (g == 0) {
+      float r = 0.f;
 #pragma unroll
-  for (int c = 0; c < CPT; ++c) acc[c] = 0.f;
+      for (int x = 0; x < G; ++x) r += part[x][c];
+      sum_s[c] = r;
+    }
+    cluster.sync();
+    if (g == 0) {
+      float r = 0.f;
+      for (int x = 0; x < n_cta; ++x) r += cluster.map_shared_rank(sum_s, x)[c];
+      mean_s[c] = r / (float)Nk;
+    }
+    __syncthreads();
+  }
+
+  // ---- this CTA's share of C_K.  Thread (ty, tx) owns rows and columns 4 ty + r (+ 64), 4 tx + c (+ 64).
+  float2 acc[T][T / 2];
+#pragma unroll
+  for (int r = 0; r < T; ++r)
+#pragma unroll
+    for (int c = 0; c < T / 2; ++c) acc[r][c] = make_float2(0.f, 0.f);
   for (int j0 = j_begin; j0 < j_end; j0 += JT) {
     const int nj = min(JT, j_end - j0);
-    for (int e = threadIdx.x; e < nj * D; e += 256) {
-      const int jj = e / D, c = e % D;
-      xs[jj][c] = kc[(size_t)(j0 + jj) * D + c] - mk[c];
+    const float4* src = reinterpret_cast<const float4*>(kc + (size_t)j0 * D);
+#pragma unroll 4
+    for (int e = tid; e < nj * (D / 4); e += 256) {
+      float4 x = src[e];
+      const float4 m = *reinterpret_cast<const float4*>(mean_s + (e % (D / 4)) * 4);
+      x.x -= m.x; x.y -= m.y; x.z -= m.z; x.w -= m.w;
+      reinterpret_cast<float4*>(work)[e] = x;
     }
     __syncthreads();
+#pragma unroll 2
     for (int jj = 0; jj < nj; ++jj) {
-      const float xr = xs[jj][r];
+      const float* x = work + jj * D;
+      float a[T], b[T];
 #pragma unroll
-      for (int c = 0; c < CPT; ++c) acc[c] = fmaf(xr, xs[jj][c0 + c], acc[c]);
+      for (int h = 0; h < T / 4; ++h) {
+        *reinterpret_cast<float4*>(a + 4 * h) = *reinterpret_cast<const float4*>(x + 64 * h + 4 * ty);
+        *reinterpret_cast<float4*>(b + 4 * h) = *reinterpret_cast<const float4*>(x + 64 * h + 4 * tx);
+      }
+#pragma unroll
+      for (int r = 0; r < T; ++r)
+#pragma unroll
+        for (int c = 0; c < T / 2; ++c)
+          acc[r][c] = __ffma2_rn(make_float2(a[r], a[r]), make_float2(b[2 * c], b[2 * c + 1]), acc[r][c]);
     }
     __syncthreads();
   }
-  float* cov = ws.covk + (((size_t)blockIdx.z * gridDim.y + bh) * D + r) * D + c0;
+  const float inv = 1.f / (float)Nk;
 #pragma unroll
-  for (int c = 0; c < CPT; ++c) cov[c] = acc[c] / (float)Nk;
-}
+  for (int r = 0; r < T; ++r)
+#pragma unroll
+    for (int h = 0; h < T / 4; ++h) {
+      const float2 lo = acc[r][2 * h], hi = acc[r][2 * h + 1];
+      *reinterpret_cast<float4*>(cov + (size_t)((r / 4) * 64 + 4 * ty + r % 4) * D + 64 * h + 4 * tx) =
+          make_float4(lo.x * inv, lo.y * inv, hi.x * inv, hi.y * inv);
+    }
+  if (n_cta > 1) {
+    cluster.sync();
+    // add the partial matrices, one strip per CTA, then gather the strips
+    constexpr int kPieces = D * D / 4;
+    const int per = ceil_div(kPieces, n_cta);
+    const int e0 = min(kPieces, rank * per), e1 = min(kPieces, e0 + per);
+    for (int e = e0 + tid; e < e1; e += 256) {
+      float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+      for (int x = 0; x < n_cta; ++x) {
+        const float4 y = reinterpret_cast<const float4*>(cluster.map_shared_rank(cov, x))[e];
+        r.x += y.x; r.y += y.y; r.z += y.z; r.w += y.w;
+      }
+      reinterpret_cast<float4*>(work)[e - e0] = r;
+    }
+    cluster.sync();
+#pragma unroll 4
+    for (int e = tid; e < kPieces; e += 256)
+      reinterpret_cast<float4*>(cov)[e] = reinterpret_cast<const float4*>(cluster.map_shared_rank(work, e / per))[e % per];
+    cluster.sync();                              // the strips are read: `work` is free again, and a CTA may leave
+  } else {
+    __syncthreads();
+  }
 
-// Per-query-block statistics and threshold (Eq. 4, Eq. 5):
-//   mu_i = s * Qbar_i . m_K,   sigma_i^2 = s^2 * Qbar_i C_K Qbar_i^T,   tau_i = mu_i + beta sigma_i.
-// Grid (ceil(Nq / 64), BH).  A CTA stages C_K and 64 pooled queries in shared memory and forms
-// Y = Qbar C_K as a register-tiled product (thread (rg, cg): 4 query blocks x 8 channels); the
-// quadratic form is the row sum of Y o Qbar, reduced over the 16 threads of a query-block group.
-template <int D>
-__global__ void __launch_bounds__(256) tau_kernel(WsPtrs ws, int Nq, float scale, float beta) {
-  extern __shared__ float smem_f[];
-  constexpr int QT = 64;                         // query blocks per CTA
-  constexpr int CPT = D / 16;                    // channels per thread (8 or 4)
-  float* cov_s = smem_f;                         // [D][D]
-  float* q_s = smem_f + D * D;                   // [QT][D + 1]
-  constexpr int QLD = D + 1;
-  const int bh = blockIdx.y, i0 = blockIdx.x * QT;
-  const size_t slice_stride = (size_t)gridDim.y * D * D;
-  const float* cov = ws.covk + (size_t)bh * D * D;
-  for (int e = threadIdx.x; e < D * D / 4; e += 256) {
-    float4 a = reinterpret_cast<const float4*>(cov)[e];
+  // ---- Y = Qbar C_K and the row sums of Y o Qbar; thread (ty, tx) owns query blocks ty + 16 a and columns
+  //      4 tx + c (+ 64)
+  constexpr int LD = D + 4;
+  const int per_q = ceil_div(Nq, n_cta);
+  const int i_begin = min(Nq, rank * per_q), i_end = min(Nq, i_begin + per_q);
+  auto rows = [&](auto a_c, int i0) {
+    constexpr int A = decltype(a_c)::value;
+    const int nq = min(16 * A, i_end - i0);
+    const float4* src = reinterpret_cast<const float4*>(ws.qbar + ((size_t)bh * Nq + i0) * D);
+#pragma unroll 4
+    for (int e = tid; e < 16 * A * (D / 4); e += 256)
+      *reinterpret_cast<float4*>(work + (e / (D / 4)) * LD + (e % (D / 4)) * 4) =
+          e / (D / 4) < nq ? src[e] : make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+    float2 y[A][T / 2];
 #pragma unroll
-    for (int sl = 1; sl < kCovSlices; ++sl) {
-      const float4 b = reinterpret_cast<const float4*>(cov + sl * slice_stride)[e];
-      a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
-    }
-    reinterpret_cast<float4*>(cov_s)[e] = a;
-  }
-  for (int e = threadIdx.x; e < QT * D; e += 256) {
-    const int rq = e / D, c = e % D;
-    q_s[rq * QLD + c] = (i0 + rq < Nq) ? ws.qbar[((size_t)bh * Nq + i0 + rq) * D + c] : 0.f;
-  }
-  __syncthreads();
-  const int rg = threadIdx.x / 16, cg = threadIdx.x % 16;
-  const int c0 = cg * CPT;
-  float y[4][CPT];
+    for (int a = 0; a < A; ++a)
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+      for (int c = 0; c < T / 2; ++c) y[a][c] = make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (int k = 0; k < D; k += 4) {
+      float q[A][4];
 #pragma unroll
-    for (int c = 0; c < CPT; ++c) y[a][c] = 0.f;
-  for (int k = 0; k < D; ++k) {
-    float qa[4], cb[CPT];
+      for (int a = 0; a < A; ++a)
+        *reinterpret_cast<float4*>(q[a]) = *reinterpret_cast<const float4*>(work + (ty + 16 * a) * LD + k);
 #pragma unroll
-    for (int a = 0; a < 4; ++a) qa[a] = q_s[(rg * 4 + a) * QLD + k];
+      for (int kk = 0; kk < 4; ++kk) {
+        float b[T];
 #pragma unroll
-    for (int c = 0; c < CPT; ++c) cb[c] = cov_s[k * D + c0 + c];
+        for (int h = 0; h < T / 4; ++h)
+          *reinterpret_cast<float4*>(b + 4 * h) = *reinterpret_cast<const float4*>(cov + (k + kk) * D + 64 * h + 4 * tx);
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+        for (int a = 0; a < A; ++a)
 #pragma unroll
-      for (int c = 0; c < CPT; ++c) y[a][c] = fmaf(qa[a], cb[c], y[a][c]);
-  }
-  const float* mk = ws.mk + (size_t)bh * D;
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    float quad = 0.f, dotm = 0.f;
-#pragma unroll
-    for (int c = 0; c < CPT; ++c) {
-      const float qv = q_s[(rg * 4 + a) * QLD + c0 + c];
-      quad = fmaf(y[a][c], qv, quad);
-      dotm = fmaf(qv, mk[c0 + c], dotm);
+          for (int c = 0; c < T / 2; ++c)
+            y[a][c] = __ffma2_rn(make_float2(q[a][kk], q[a][kk]), make_float2(b[2 * c], b[2 * c + 1]), y[a][c]);
+      }
     }
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) {
-      quad += __shfl_xor_sync(0xffffffffu, quad, o);
-      dotm += __shfl_xor_sync(0xffffffffu, dotm, o);
+    for (int a = 0; a < A; ++a) {
+      float quad = 0.f, dotm = 0.f;
+#pragma unroll
+      for (int c = 0; c < T; ++c) {
+        const int at = (c / 4) * 64 + 4 * tx + c % 4;
+        const float qv = work[(ty + 16 * a) * LD + at];
+        quad = fmaf((c & 1) ? y[a][c / 2].y : y[a][c / 2].x, qv, quad);
+        dotm = fmaf(qv, mean_s[at], dotm);
+      }
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) {
+        quad += __shfl_xor_sync(0xffffffffu, quad, o);
+        dotm += __shfl_xor_sync(0xffffffffu, dotm, o);
+      }
+      const int i = i0 + ty + 16 * a;
+      if (tx == 0 && i < i_end)
+        store_threshold(ws, (size_t)bh * Nq + i, scale * dotm, scale * sqrtf(fmaxf(quad, 0.f)), beta);
     }
-    const int i = i0 + rg * 4 + a;
-    if (cg == 0 && i < Nq) {
-      const float mu = scale * dotm;
-      const float sigma = scale * sqrtf(fmaxf(quad, 0.f));
-      float tau;
-      if (isinf(beta)) tau = beta;               // +inf: route nothing, -inf: route everything
-      else tau = fmaf(beta, sigma, mu);
-      const size_t o = (size_t)bh * Nq + i;
-      ws.mu[o] = mu;
-      ws.sigma[o] = sigma;
-      ws.tau[o] = tau;
+    __syncthreads();
+  };
+  for (int i0 = i_begin; i0 < i_end;) {          // few blocks left: a step of 32 does
+    if (i_end - i0 > 32) {
+      rows(std::integral_constant<int, kMomentRows / 16>{}, i0);
+      i0 += kMomentRows;
+    } else {
+      rows(std::integral_constant<int, 2>{}, i0);
+      i0 += 32;
     }
   }
 }
@@ -243,24 +409,23 @@ __global__ void __launch_bounds__(256) tau_kernel(WsPtrs ws, int Nq, float scale
 }  // namespace
 
 cudaError_t launch_pool(const Problem& p, const __nv_bfloat16* q, const __nv_bfloat16* k,
-                        const __nv_bfloat16* v, const WsPtrs& ws, cudaStream_t stream, int* n_launches) {
+                        const __nv_bfloat16* v, const WsPtrs& ws, int zero_from, cudaStream_t stream, int* n_launches) {
   const int first_kind = q ? 0 : 1;
   const long long blocks = (long long)p.BH * ((q ? p.Nq : 0) + 2LL * p.Nk);
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   if (p.d == 128)
     pool_kernel<128><<<(unsigned)blocks, kPoolThreads, 0, stream>>>(q, k, v, ws, p.st, p.N, p.block_q, p.block_k,
-                                                                      p.Nq, p.Nk, first_kind);
+                                                                      p.Nq, p.Nk, first_kind, zero_from);
   else
     pool_kernel<64><<<(unsigned)blocks, kPoolThreads, 0, stream>>>(q, k, v, ws, p.st, p.N, p.block_q, p.block_k,
-                                                                     p.Nq, p.Nk, first_kind);
+                                                                     p.Nq, p.Nk, first_kind, zero_from);
   if (n_launches) *n_launches += 1;
   return cudaGetLastError();
 }
 
 // Diagonal estimator (appendix, Eq. appendix_diagonal_threshold): only the per-channel variance of
 // the pooled keys is kept, v_K = mean_j KC_j o KC_j - m_K o m_K (computed in centred form), and
-// sigma_i^2 = s^2 (Qbar_i o Qbar_i) . v_K.  One CTA per (batch, head) writes m_K and v_K (v_K goes
-// to the first D floats of the head's second-moment area).
+// sigma_i^2 = s^2 (Qbar_i o Qbar_i) . v_K.  One CTA per (batch, head) writes m_K and v_K.
 template <int D>
 __global__ void __launch_bounds__(4 * D) key_diag_kernel(WsPtrs ws, int Nk) {
   __shared__ float part[4][D];
@@ -284,7 +449,7 @@ __global__ void __launch_bounds__(4 * D) key_diag_kernel(WsPtrs ws, int Nk) {
   __syncthreads();
   if (grp == 0) {
     ws.mk[(size_t)bh * D + c] = m;
-    ws.covk[(size_t)bh * D * D + c] = ((part[0][c] + part[1][c]) + (part[2][c] + part[3][c])) / (float)Nk;
+    ws.vk[(size_t)bh * D + c] = ((part[0][c] + part[1][c]) + (part[2][c] + part[3][c])) / (float)Nk;
   }
 }
 
@@ -296,7 +461,7 @@ __global__ void __launch_bounds__(256) tau_diag_kernel(WsPtrs ws, int Nq, float 
   if (i >= Nq) return;
   const float* qb = ws.qbar + ((size_t)bh * Nq + i) * D;
   const float* mk = ws.mk + (size_t)bh * D;
-  const float* vk = ws.covk + (size_t)bh * D * D;
+  const float* vk = ws.vk + (size_t)bh * D;
   float quad = 0.f, dotm = 0.f;
 #pragma unroll
   for (int c = lane; c < D; c += 32) {
@@ -310,31 +475,53 @@ __global__ void __launch_bounds__(256) tau_diag_kernel(WsPtrs ws, int Nq, float 
     dotm += __shfl_xor_sync(0xffffffffu, dotm, o);
   }
   if (lane == 0) {
-    const float mu = scale * dotm;
-    const float sigma = scale * sqrtf(fmaxf(quad, 0.f));
-    const size_t o = (size_t)bh * Nq + i;
-    ws.mu[o] = mu;
-    ws.sigma[o] = sigma;
-    ws.tau[o] = isinf(beta) ? beta : fmaf(beta, sigma, mu);
+    store_threshold(ws, (size_t)bh * Nq + i, scale * dotm, scale * sqrtf(fmaxf(quad, 0.f)), beta);
   }
 }
 
 template <int D>
 static cudaError_t thresholds_impl(const Problem& p, const WsPtrs& ws, cudaStream_t stream, int* n_launches) {
-  if (p.estimator == SOL_EST_DIAGONAL) {
+  const bool diag = p.estimator == SOL_EST_DIAGONAL;
+  if (p.Nk <= kSmallKeys) {
+    const size_t smem = sizeof(float) * p.Nk * (D + 4);
+    auto kernel = diag ? thresholds_small_kernel<D, true> : thresholds_small_kernel<D, false>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kernel<<<dim3(ceil_div(p.Nq, kSmallRows), p.BH), 256, smem, stream>>>(ws, p.Nq, p.Nk, p.scale, p.beta);
+    if (n_launches) *n_launches += 1;
+    return cudaGetLastError();
+  }
+  if (diag) {
     key_diag_kernel<D><<<p.BH, 4 * D, 0, stream>>>(ws, p.Nk);
     tau_diag_kernel<D><<<dim3(ceil_div(p.Nq, 8), p.BH), 256, 0, stream>>>(ws, p.Nq, p.scale, p.beta);
     if (n_launches) *n_launches += 2;
     return cudaGetLastError();
   }
-  key_mean_kernel<D><<<p.BH, 4 * D, 0, stream>>>(ws, p.Nk);
-  key_cov_kernel<D><<<dim3(D / 16, p.BH, kCovSlices), 256, 0, stream>>>(ws, p.Nk);
-  const size_t smem = sizeof(float) * (D * D + 64 * (D + 1));
-  cudaError_t e = cudaFuncSetAttribute(tau_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // one cluster per head, as large as two CTAs per SM allow (8 at most): a second wave would cost a whole pass
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  tau_kernel<D><<<dim3(ceil_div(p.Nq, 64), p.BH), 256, smem, stream>>>(ws, p.Nq, p.scale, p.beta);
-  if (n_launches) *n_launches += 3;
-  return cudaGetLastError();
+  const int fit = 2 * sms / p.BH;
+  const int n_cta = fit < 1 ? 1 : (fit > 8 ? 8 : fit);
+  const size_t smem = moments_smem<D>();
+  e = cudaFuncSetAttribute(thresholds_moments_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(n_cta, p.BH);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = n_cta;
+  attr.val.clusterDim.y = 1;
+  attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  e = cudaLaunchKernelEx(&cfg, thresholds_moments_kernel<D>, ws, p.Nq, p.Nk, p.scale, p.beta);
+  if (n_launches) *n_launches += 1;
+  return e;
 }
 
 cudaError_t launch_thresholds(const Problem& p, const WsPtrs& ws, cudaStream_t stream, int* n_launches) {
