@@ -188,9 +188,12 @@ __device__ void router_role(Shared<C>& sm, const Params& p, int lane) {
   PROF_DECL
   if (lane == 0) CTATRACE(0, prof::gtimer());
   while (alive) {
-    int w = 0;
-    if (lane == 0) w = atomicAdd(p.status + kStatusTileCounter, 1);
-    w = __shfl_sync(full, w, 0);
+    // the first work item is the CTA's own number (a round trip to memory less at the start), then the counter's
+    int w = (int)blockIdx.x;
+    if (n_item > 0) {
+      if (lane == 0) w = (int)gridDim.x + atomicAdd(p.status + kStatusTileCounter, 1);
+      w = __shfl_sync(full, w, 0);
+    }
     if (w >= p.total_work) break;
     if (lane == 0) ITRACE(n_item, 0);
     const int bh = w / p.Nq, i = w - bh * p.Nq;
@@ -855,6 +858,7 @@ fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
+  kernel_wait();
 
   if (warp < 8) {
     softmax_role<C>(sm, p, tmem, warp / 4, warp % 4, lane);
@@ -882,10 +886,7 @@ cudaError_t launch_instance(const Problem& p, const Maps& m, const Params& prm, 
   // the pre-pass variant is a kernel of its own, so that the in-kernel router's code is what it is without it
   auto kernel = p.routing == SOL_ROUTING_PREPASS && p.mode != SOL_MODE_DENSE ? fwd_sm100_kernel<C, true>
                                                                             : fwd_sm100_kernel<C, false>;
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  kernel<<<grid, kThreads, smem, stream>>>(m.q, m.k, m.v, m.kc, m.vm, prm);
-  return cudaGetLastError();
+  return launch_after(kernel, dim3(grid), kThreads, smem, 0, stream, m.q, m.k, m.v, m.kc, m.vm, prm);
 }
 
 }  // namespace

@@ -137,12 +137,32 @@ __device__ void router_role(Shared<C>& sm, const Params& p, int lane) {
   const float bias_last = log2f((float)(p.N - (p.Nk - 1) * kBlk)) * inv_sl2;     // ... and of the ragged last one
   bool alive = true;
   while (alive) {
-    int w = 0;
-    if (lane == 0) w = atomicAdd(p.status + kStatusTileCounter, 1);
-    w = __shfl_sync(full, w, 0);
+    // the first work item is the CTA's own number (a round trip to memory less at the start), then the counter's
+    int w = (int)blockIdx.x;
+    if (n_item > 0) {
+      if (lane == 0) w = (int)gridDim.x + atomicAdd(p.status + kStatusTileCounter, 1);
+      w = __shfl_sync(full, w, 0);
+    }
     if (w >= p.total_work) break;
     const int bh = w / p.items_per_head;
     const int i0 = (w - bh * p.items_per_head) * p.per_item;
+    const float* kc_head = p.kc + (size_t)bh * p.Nk * kD;
+    // Bulk-copy kGroup pooled keys (contiguous in memory) into a staging buffer; the copy of the next
+    // ones is in flight while these are scored.
+    auto stage_group = [&](int jb) {
+      if (!score || jb >= p.Nk) return;
+      __syncwarp();                                  // every lane is done reading this buffer
+      if (lane == 0) {
+        const uint32_t buf = n_copy & 1;
+        const uint32_t bytes = (uint32_t)min(kGroup, p.Nk - jb) * kD * 4;
+        fence_proxy_async_smem();
+        mbar_arrive_expect_tx(&sm.kc_full[buf], bytes);
+        bulk_load_1d(sm.kc_stage[buf], kc_head + (size_t)jb * kD, bytes, &sm.kc_full[buf]);
+      }
+      ++n_copy;
+    };
+    stage_group(0);
+    stage_group(kGroup);
     // query block u of the item: the streams take one block each until a full item gives them two
     const int step = p.per_item == kNQ ? 1 : kSub;
     int valid = 0;
@@ -164,27 +184,10 @@ __device__ void router_role(Shared<C>& sm, const Params& p, int lane) {
       }
     }
     __syncwarp();
-    const float* kc_head = p.kc + (size_t)bh * p.Nk * kD;
     const size_t row0 = (size_t)bh * p.Nq + i0;      // counts / mask row of block u: row0 + u / step
     int count[kNQ];
 #pragma unroll
     for (int u = 0; u < kNQ; ++u) count[u] = 0;
-    // Bulk-copy kGroup pooled keys (contiguous in memory) into a staging buffer; the copy of the next
-    // ones is in flight while these are scored.
-    auto stage_group = [&](int jb) {
-      if (!score || jb >= p.Nk) return;
-      __syncwarp();                                  // every lane is done reading this buffer
-      if (lane == 0) {
-        const uint32_t buf = n_copy & 1;
-        const uint32_t bytes = (uint32_t)min(kGroup, p.Nk - jb) * kD * 4;
-        fence_proxy_async_smem();
-        mbar_arrive_expect_tx(&sm.kc_full[buf], bytes);
-        bulk_load_1d(sm.kc_stage[buf], kc_head + (size_t)jb * kD, bytes, &sm.kc_full[buf]);
-      }
-      ++n_copy;
-    };
-    stage_group(0);
-    stage_group(kGroup);
     for (int t = 0; t < n_chunks; ++t) {
       Record& rec = sm.rec[n_rec % kRecords];
       if (!WAIT(&sm.rec_empty[n_rec % kRecords], ((n_rec / kRecords) & 1) ^ 1)) {
@@ -894,6 +897,7 @@ fwd_sm100_b64_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
+  kernel_wait();
 
   if (warp < 8) {
     softmax_role<C>(sm, p, tmem, warp / 4, warp % 4, lane);
@@ -914,10 +918,7 @@ cudaError_t launch_instance(const Problem& p, const Maps& m, const Params& prm, 
   const size_t smem = 1024 + 2 * C::kQBytes + 2 * kStages * C::kTileBytes + sizeof(Shared<C>);
   auto kernel = p.routing == SOL_ROUTING_PREPASS && p.mode != SOL_MODE_DENSE ? fwd_sm100_b64_kernel<C, true>
                                                                             : fwd_sm100_b64_kernel<C, false>;
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  kernel<<<grid, kThreads, smem, stream>>>(m.q, m.k, m.v, m.kc, m.vm, prm);
-  return cudaGetLastError();
+  return launch_after(kernel, dim3(grid), kThreads, smem, 0, stream, m.q, m.k, m.v, m.kc, m.vm, prm);
 }
 
 }  // namespace

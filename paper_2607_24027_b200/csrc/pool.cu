@@ -138,6 +138,8 @@ __global__ void __launch_bounds__(256) thresholds_small_kernel(WsPtrs ws, int Nq
   const float* kc = ws.kc + (size_t)bh * Nk * D;
   const float* qb = ws.qbar + ((size_t)bh * Nq + i0) * D;
   const int nq = min(kSmallRows, Nq - i0);
+  kernel_wait();
+  kernel_release();
 #pragma unroll 4
   for (int e = tid; e < Nk * (D / 4); e += 256)
     *reinterpret_cast<float4*>(ks + (e / (D / 4)) * LD + (e % (D / 4)) * 4) = reinterpret_cast<const float4*>(kc)[e];
@@ -218,20 +220,21 @@ __global__ void __launch_bounds__(256) thresholds_small_kernel(WsPtrs ws, int Nq
 // A thread-block cluster takes one head.  Each CTA sums its share of the keys, first for the mean, then for a
 // partial C_K in registers (256 threads, 8 x 8 or 4 x 4 each); the partial sums are added through distributed
 // shared memory in rank order (bit-stable run to run), every CTA gathers the whole C_K and forms Y = Qbar C_K for
-// its share of the query blocks.  FMA-bound: 1.5 GFLOP at 40 heads x 591 blocks, d = 128, 92 us, where
-// three kernels (mean on 40 CTAs; C_K with one shared-memory operand per FMA; quadratic form) took 198 us.
-constexpr int kMomentRows = 80;                  // query blocks per step: 5 for each of 16 thread rows
+// its share of the query blocks.  A share of up to 88 keys stays in shared memory between the two passes, and up to
+// 88 query blocks are one step: with two CTAs per SM that is the largest `work` area there is room for, and what 40
+// heads of 591 blocks give a CTA of a cluster of 7.  1.5 GFLOP at that size, 60 us; three kernels (mean on 40
+// CTAs; C_K with one shared-memory operand per FMA; quadratic form) took 198 us.
+constexpr int kMomentRows = 88;
 
 template <int D>
-constexpr size_t moments_smem() {                // C_K, then (in turn) staged keys / a reduced strip / pooled queries
-  constexpr size_t work = sizeof(float) * kMomentRows * (D + 4), strip = sizeof(float) * D * D / 2;
+constexpr size_t moments_smem() {                // C_K, then (in turn) keys / a reduced strip / pooled queries
+  constexpr size_t work = sizeof(float) * kMomentRows * D, strip = sizeof(float) * D * D / 2;
   return sizeof(float) * D * D + (work > strip ? work : strip);
 }
 
 template <int D>
 __global__ void __launch_bounds__(256, 2) thresholds_moments_kernel(WsPtrs ws, int Nq, int Nk, float scale, float beta) {
   constexpr int T = D / 16;                      // C_K rows and columns per thread (8 or 4)
-  constexpr int JT = 32;                         // keys staged per step
   constexpr int G = 256 / D;
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
@@ -246,24 +249,41 @@ __global__ void __launch_bounds__(256, 2) thresholds_moments_kernel(WsPtrs ws, i
   const int per_k = ceil_div(Nk, n_cta);
   const int j_begin = min(Nk, rank * per_k), j_end = min(Nk, j_begin + per_k);
 
+  // copies n rows of D floats to `work`
+  auto stage = [&](const float* src, int n) {
+#pragma unroll 4
+    for (int e = tid; e < n * (D / 4); e += 256)
+      reinterpret_cast<float4*>(work)[e] = reinterpret_cast<const float4*>(src)[e];
+  };
+  kernel_wait();
+  const bool resident = j_end - j_begin <= kMomentRows;
+
   // ---- m_K
   {
+    if (resident) {
+      stage(kc + (size_t)j_begin * D, j_end - j_begin);
+      __syncthreads();
+    }
+    const float* x = resident ? work : kc + (size_t)j_begin * D;
     const int c = tid % D, g = tid / D;
     float s = 0.f;
 #pragma unroll 8
-    for (int j = j_begin + g; j < j_end; j += G) s += kc[(size_t)j * D + c];
+    for (int j = g; j < j_end - j_begin; j += G) s += x[(size_t)j * D + c];
     part[g][c] = s;
     __syncthreads();
     if (g == 0) {
       float r = 0.f;
 #pragma unroll
-      for (int x = 0; x < G; ++x) r += part[x][c];
+      for (int y = 0; y < G; ++y) r += part[y][c];
       sum_s[c] = r;
     }
     cluster.sync();
     if (g == 0) {
-      float r = 0.f;
-      for (int x = 0; x < n_cta; ++x) r += cluster.map_shared_rank(sum_s, x)[c];
+      float other[8], r = 0.f;
+#pragma unroll
+      for (int y = 0; y < 8; ++y) other[y] = y < n_cta ? cluster.map_shared_rank(sum_s, y)[c] : 0.f;
+#pragma unroll
+      for (int y = 0; y < 8; ++y) r += other[y];
       mean_s[c] = r / (float)Nk;
     }
     __syncthreads();
@@ -275,12 +295,14 @@ __global__ void __launch_bounds__(256, 2) thresholds_moments_kernel(WsPtrs ws, i
   for (int r = 0; r < T; ++r)
 #pragma unroll
     for (int c = 0; c < T / 2; ++c) acc[r][c] = make_float2(0.f, 0.f);
-  for (int j0 = j_begin; j0 < j_end; j0 += JT) {
-    const int nj = min(JT, j_end - j0);
-    const float4* src = reinterpret_cast<const float4*>(kc + (size_t)j0 * D);
-#pragma unroll 4
+  for (int j0 = j_begin; j0 < j_end; j0 += kMomentRows) {
+    const int nj = min(kMomentRows, j_end - j0);
+    if (!resident) {
+      stage(kc + (size_t)j0 * D, nj);
+      __syncthreads();
+    }
     for (int e = tid; e < nj * (D / 4); e += 256) {
-      float4 x = src[e];
+      float4 x = reinterpret_cast<float4*>(work)[e];
       const float4 m = *reinterpret_cast<const float4*>(mean_s + (e % (D / 4)) * 4);
       x.x -= m.x; x.y -= m.y; x.z -= m.z; x.w -= m.w;
       reinterpret_cast<float4*>(work)[e] = x;
@@ -319,16 +341,16 @@ __global__ void __launch_bounds__(256, 2) thresholds_moments_kernel(WsPtrs ws, i
     const int per = ceil_div(kPieces, n_cta);
     const int e0 = min(kPieces, rank * per), e1 = min(kPieces, e0 + per);
     for (int e = e0 + tid; e < e1; e += 256) {
-      float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-      for (int x = 0; x < n_cta; ++x) {
-        const float4 y = reinterpret_cast<const float4*>(cluster.map_shared_rank(cov, x))[e];
-        r.x += y.x; r.y += y.y; r.z += y.z; r.w += y.w;
-      }
+      float4 y[8], r = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int x = 0; x < 8; ++x)
+        y[x] = x < n_cta ? reinterpret_cast<const float4*>(cluster.map_shared_rank(cov, x))[e] : r;
+#pragma unroll
+      for (int x = 0; x < 8; ++x) { r.x += y[x].x; r.y += y[x].y; r.z += y[x].z; r.w += y[x].w; }
       reinterpret_cast<float4*>(work)[e - e0] = r;
     }
     cluster.sync();
-#pragma unroll 4
+#pragma unroll 8
     for (int e = tid; e < kPieces; e += 256)
       reinterpret_cast<float4*>(cov)[e] = reinterpret_cast<const float4*>(cluster.map_shared_rank(work, e / per))[e % per];
     cluster.sync();                              // the strips are read: `work` is free again, and a CTA may leave
@@ -338,18 +360,16 @@ __global__ void __launch_bounds__(256, 2) thresholds_moments_kernel(WsPtrs ws, i
 
   // ---- Y = Qbar C_K and the row sums of Y o Qbar; thread (ty, tx) owns query blocks ty + 16 a and columns
   //      4 tx + c (+ 64)
-  constexpr int LD = D + 4;
   const int per_q = ceil_div(Nq, n_cta);
   const int i_begin = min(Nq, rank * per_q), i_end = min(Nq, i_begin + per_q);
   auto rows = [&](auto a_c, int i0) {
     constexpr int A = decltype(a_c)::value;
-    const int nq = min(16 * A, i_end - i0);
-    const float4* src = reinterpret_cast<const float4*>(ws.qbar + ((size_t)bh * Nq + i0) * D);
-#pragma unroll 4
-    for (int e = tid; e < 16 * A * (D / 4); e += 256)
-      *reinterpret_cast<float4*>(work + (e / (D / 4)) * LD + (e % (D / 4)) * 4) =
-          e / (D / 4) < nq ? src[e] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const int nq = min(min(16 * A, kMomentRows), i_end - i0);
+    stage(ws.qbar + ((size_t)bh * Nq + i0) * D, nq);
     __syncthreads();
+    const float* q_row[A];                       // (rows past the last repeat it and are not stored)
+#pragma unroll
+    for (int a = 0; a < A; ++a) q_row[a] = work + min(ty + 16 * a, nq - 1) * D;
     float2 y[A][T / 2];
 #pragma unroll
     for (int a = 0; a < A; ++a)
@@ -360,7 +380,7 @@ __global__ void __launch_bounds__(256, 2) thresholds_moments_kernel(WsPtrs ws, i
       float q[A][4];
 #pragma unroll
       for (int a = 0; a < A; ++a)
-        *reinterpret_cast<float4*>(q[a]) = *reinterpret_cast<const float4*>(work + (ty + 16 * a) * LD + k);
+        *reinterpret_cast<float4*>(q[a]) = *reinterpret_cast<const float4*>(q_row[a] + k);
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk) {
         float b[T];
@@ -380,7 +400,7 @@ __global__ void __launch_bounds__(256, 2) thresholds_moments_kernel(WsPtrs ws, i
 #pragma unroll
       for (int c = 0; c < T; ++c) {
         const int at = (c / 4) * 64 + 4 * tx + c % 4;
-        const float qv = work[(ty + 16 * a) * LD + at];
+        const float qv = q_row[a][at];
         quad = fmaf((c & 1) ? y[a][c / 2].y : y[a][c / 2].x, qv, quad);
         dotm = fmaf(qv, mean_s[at], dotm);
       }
@@ -389,16 +409,19 @@ __global__ void __launch_bounds__(256, 2) thresholds_moments_kernel(WsPtrs ws, i
         quad += __shfl_xor_sync(0xffffffffu, quad, o);
         dotm += __shfl_xor_sync(0xffffffffu, dotm, o);
       }
-      const int i = i0 + ty + 16 * a;
-      if (tx == 0 && i < i_end)
-        store_threshold(ws, (size_t)bh * Nq + i, scale * dotm, scale * sqrtf(fmaxf(quad, 0.f)), beta);
+      if (tx == 0 && ty + 16 * a < nq)
+        store_threshold(ws, (size_t)bh * Nq + i0 + ty + 16 * a, scale * dotm, scale * sqrtf(fmaxf(quad, 0.f)), beta);
     }
     __syncthreads();
   };
-  for (int i0 = i_begin; i0 < i_end;) {          // few blocks left: a step of 32 does
-    if (i_end - i0 > 32) {
-      rows(std::integral_constant<int, kMomentRows / 16>{}, i0);
+  for (int i0 = i_begin; i0 < i_end;) {          // a step is as short as what is left
+    const int left = i_end - i0;
+    if (left > 64) {
+      rows(std::integral_constant<int, 6>{}, i0);
       i0 += kMomentRows;
+    } else if (left > 32) {
+      rows(std::integral_constant<int, 4>{}, i0);
+      i0 += 64;
     } else {
       rows(std::integral_constant<int, 2>{}, i0);
       i0 += 32;
@@ -483,13 +506,10 @@ template <int D>
 static cudaError_t thresholds_impl(const Problem& p, const WsPtrs& ws, cudaStream_t stream, int* n_launches) {
   const bool diag = p.estimator == SOL_EST_DIAGONAL;
   if (p.Nk <= kSmallKeys) {
-    const size_t smem = sizeof(float) * p.Nk * (D + 4);
-    auto kernel = diag ? thresholds_small_kernel<D, true> : thresholds_small_kernel<D, false>;
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kernel<<<dim3(ceil_div(p.Nq, kSmallRows), p.BH), 256, smem, stream>>>(ws, p.Nq, p.Nk, p.scale, p.beta);
     if (n_launches) *n_launches += 1;
-    return cudaGetLastError();
+    return launch_after(diag ? thresholds_small_kernel<D, true> : thresholds_small_kernel<D, false>,
+                        dim3(ceil_div(p.Nq, kSmallRows), p.BH), 256, sizeof(float) * p.Nk * (D + 4), 0, stream, ws, p.Nq,
+                        p.Nk, p.scale, p.beta);
   }
   if (diag) {
     key_diag_kernel<D><<<p.BH, 4 * D, 0, stream>>>(ws, p.Nk);
@@ -497,31 +517,18 @@ static cudaError_t thresholds_impl(const Problem& p, const WsPtrs& ws, cudaStrea
     if (n_launches) *n_launches += 2;
     return cudaGetLastError();
   }
-  // one cluster per head, as large as two CTAs per SM allow (8 at most): a second wave would cost a whole pass
+  // One cluster per head, as large as leaves every CTA an SM of its own with room for the clusters to be packed
+  // into GPCs: two CTAs on an SM share its FMA pipes and take twice as long.  40 heads x 591 blocks: clusters of 2 / 3 /
+  // 4 / 7 take 80 / 60 / 82 / 77 us; 24 heads x 300: 4 / 5 / 6 take 27 / 24 / 38 us.
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const int fit = 2 * sms / p.BH;
+  const int fit = sms * 17 / 20 / p.BH;
   const int n_cta = fit < 1 ? 1 : (fit > 8 ? 8 : fit);
-  const size_t smem = moments_smem<D>();
-  e = cudaFuncSetAttribute(thresholds_moments_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(n_cta, p.BH);
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = n_cta;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, thresholds_moments_kernel<D>, ws, p.Nq, p.Nk, p.scale, p.beta);
   if (n_launches) *n_launches += 1;
-  return e;
+  return launch_after(thresholds_moments_kernel<D>, dim3(n_cta, p.BH), 256, moments_smem<D>(), n_cta, stream, ws, p.Nq, p.Nk,
+                      p.scale, p.beta);
 }
 
 cudaError_t launch_thresholds(const Problem& p, const WsPtrs& ws, cudaStream_t stream, int* n_launches) {

@@ -26,6 +26,7 @@ __global__ void __launch_bounds__(256, 2) mask_prepass_kernel(const float* __res
   const int bh = blockIdx.z, i0 = blockIdx.y * kProxyRows, j0 = blockIdx.x * kProxyCols;
   const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
   float dot[8][4];
+  kernel_wait();
   proxy_tile<true>(qbar + ((size_t)bh * Nq + i0) * d, kc + ((size_t)bh * Nk + j0) * d, Nq - i0, Nk - j0, d, smem_f, dot);
   bool force[4];
 #pragma unroll
@@ -56,12 +57,10 @@ __global__ void __launch_bounds__(256, 2) mask_prepass_kernel(const float* __res
 
 cudaError_t launch_route_prepass(const Problem& p, const WsPtrs& ws, const float* tau, uint32_t* mask,
                                  cudaStream_t stream, int* n_launches) {
-  const cudaError_t e = cudaFuncSetAttribute(mask_prepass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kProxySmem);
-  if (e != cudaSuccess) return e;
   const dim3 grid(ceil_div(p.Nk, kProxyCols), ceil_div(p.Nq, kProxyRows), p.BH);
-  mask_prepass_kernel<<<grid, 256, kProxySmem, stream>>>(ws.qbar, ws.kc, tau, p.forced, mask, p.Nq, p.Nk, p.d, p.scale);
   if (n_launches) *n_launches += 1;
-  return cudaGetLastError();
+  return launch_after(mask_prepass_kernel, grid, 256, kProxySmem, 0, stream, ws.qbar, ws.kc, tau, p.forced, mask, p.Nq, p.Nk,
+                      p.d, p.scale);
 }
 
 }  // namespace sol
