@@ -49,14 +49,19 @@ sol_status_t host_path(HostPath* hp) {
   return SOL_OK;
 }
 
-// bytes of one tensor per group of heads on the host path (SOL_ATTN_HOST_GROUP_BYTES may change between calls)
-size_t host_group_bytes() {
-  size_t want = size_t(64) << 20;                            // about 64 MB per tensor and group
+// Bytes of one tensor per group of heads on the host path: a quarter of the tensor, so that the first group's kernels
+// start and the first output goes back while most of the input is still to come, between 4 MB (below that the four
+// copies and three launches of a group cost more than they hide) and 64 MB.  24 heads x 4096 tokens (25 MB a tensor) in
+// groups of 1 / 2 / 4 / 6 / 8 / 25 MB: 2.47 / 1.95 / 1.86 / 1.79 / 1.74 / 2.55 ms; 40 heads x 900 tokens (9 MB) in groups of
+// 0.5 / 1 / 2 / 4 / 9 MB: 1.23 / 1.02 / 0.89 / 0.69 / 1.51 ms; 24 heads x 16 000 tokens (98 MB) in groups of 24 / 64 MB: 6.06 /
+// 6.49 ms.  (SOL_ATTN_HOST_GROUP_BYTES sets the size instead; it may change between calls.)
+size_t host_group_bytes(size_t tensor_bytes) {
   if (const char* env = getenv("SOL_ATTN_HOST_GROUP_BYTES")) {
     const long long v = atoll(env);
-    if (v > 0) want = (size_t)v;
+    if (v > 0) return (size_t)v;
   }
-  return want;
+  const size_t lo = size_t(4) << 20, hi = size_t(64) << 20, quarter = tensor_bytes / 4;
+  return quarter < lo ? lo : (quarter > hi ? hi : quarter);
 }
 
 sol_status_t check_arch() { return sol::check_device_arch(); }
@@ -313,7 +318,7 @@ sol_status_t sol_attn_forward_host(const void* hq, const void* hk, const void* h
   // device on one copy stream and the previous group's output travels back on another.
   const int BH = B * H, Nq = sol::ceil_div(N, block_q);
   const size_t head_bytes = (size_t)N * d * 2;
-  const size_t want = host_group_bytes();
+  const size_t want = host_group_bytes((size_t)BH * head_bytes);
   int per = (int)((want + head_bytes - 1) / head_bytes);
   if (per < 1) per = 1;
   if (per > BH) per = BH;
