@@ -118,7 +118,8 @@ template <class... P, class... A>
 cudaError_t launch_after(void (*kernel)(P...), dim3 grid, int threads, size_t smem, int cluster, cudaStream_t stream,
                          A... args) {
   cudaError_t e = cudaSuccess;
-  if (smem > 48 * 1024) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (48 KB is the default limit for static and dynamic shared memory together)
+  if (smem > 32 * 1024) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;

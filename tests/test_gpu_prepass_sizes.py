@@ -22,9 +22,9 @@ def _pooled(BH, N, d, block, seed):
     return q, k, v
 
 
-# Nk: one block, the sizes next to the 128 of the one-pass kernel, row steps of 32 / 64 / 88 per CTA of a cluster, and
+# Nk: one block, sizes at which the one-pass kernel's shared memory is just below and above 48 KB, the sizes next to its 128, row steps of 32 / 64 / 88 per CTA of a cluster, and
 # clusters of 8, 7 (40 heads), 1 (400 heads)
-@pytest.mark.parametrize("BH,n_blocks,d", [(1, 1, 64), (3, 17, 128), (2, 128, 64), (2, 128, 128), (2, 129, 64), (2, 129, 128),
+@pytest.mark.parametrize("BH,n_blocks,d", [(1, 1, 64), (3, 17, 128), (2, 66, 128), (2, 73, 128), (2, 90, 128), (2, 92, 128), (2, 128, 64), (2, 128, 128), (2, 129, 64), (2, 129, 128),
                                            (3, 300, 128), (40, 260, 128), (40, 591, 64), (400, 130, 64), (1, 1500, 128)])
 @pytest.mark.parametrize("estimator", ["moments", "diagonal"])
 def test_thresholds(sb, BH, n_blocks, d, estimator):
