@@ -928,7 +928,7 @@ cudaError_t launch_b64(const Problem& p, const __nv_bfloat16* q, const __nv_bflo
                        long long wait_limit, int withhold_tile, cudaStream_t stream, int* n_launches) {
   Maps m;
   Params prm;
-  if (!prepare(p, q, k, v, out, ws, tau, counts, mask_out, &m, &prm)) return cudaErrorInvalidValue;
+  if (!prepare(p, q, k, v, out, ws, tau, counts, mask_out, kBlk, &m, &prm)) return cudaErrorInvalidValue;
   prm.wait_limit = wait_limit;
   prm.withhold_tile = withhold_tile;
   int sms = 0;

@@ -1,5 +1,5 @@
-// What the two tcgen05 forward kernels (fwd_sm100.cu: 128-token blocks, fwd_sm100_b64.cu: 64-token blocks)
-// have in common: launch parameters, the failure flag and a few TMEM / descriptor helpers.
+// What the tcgen05 forward kernels (fwd_sm100.cu: 128-token blocks, fwd_sm100_b64.cu: 64-token blocks,
+// fwd_sm100_dense.cu: dense mode) have in common: launch parameters, the failure flag and a few TMEM / descriptor helpers.
 #pragma once
 
 #include "common.cuh"
@@ -60,10 +60,10 @@ __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t* r) {   //
   for (int c = 0; c < N; c += 32) tmem_ld_32x32b_x32(taddr + c, *reinterpret_cast<uint32_t(*)[32]>(r + c));
 }
 
-// Tensor maps and launch parameters of one problem (everything but the work split and the test hook's state).
+// Tensor maps and launch parameters of one problem, K and V tiles of kv_rows keys (everything but the work split and the test hook's state).
 inline bool prepare(const Problem& p, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
                     __nv_bfloat16* out, const WsPtrs& ws, const float* tau, int32_t* counts, uint32_t* mask_out,
-                    Maps* m, Params* prm) {
+                    int kv_rows, Maps* m, Params* prm) {
   bool rows_inner = true, pooled_inner = true;
   auto user_map = [&](CUtensorMap* t, const void* base, int box_rows) {
     return make_tmap_bf16_4d(t, base, p.B, p.H, p.N, p.d, box_rows, p.st.row, p.st.head, p.st.batch, &rows_inner);
@@ -72,7 +72,7 @@ inline bool prepare(const Problem& p, const __nv_bfloat16* q, const __nv_bfloat1
     return make_tmap_bf16_4d(t, base, p.B, p.H, p.Nk, p.d, p.block_k, p.d, (long long)p.Nk * p.d,
                              (long long)p.H * p.Nk * p.d, &pooled_inner);
   };
-  if (!user_map(&m->q, q, kRowsQ) || !user_map(&m->k, k, p.block_k) || !user_map(&m->v, v, p.block_k) ||
+  if (!user_map(&m->q, q, kRowsQ) || !user_map(&m->k, k, kv_rows) || !user_map(&m->v, v, kv_rows) ||
       !pooled_map(&m->kc, ws.kcb) || !pooled_map(&m->vm, ws.vmb) || !pooled_inner)
     return false;
   *prm = Params{};
@@ -95,6 +95,11 @@ inline cudaError_t sm_count(int* sms) {
 cudaError_t launch_b64(const Problem& p, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
                        __nv_bfloat16* out, const WsPtrs& ws, const float* tau, int32_t* counts, uint32_t* mask_out,
                        long long wait_limit, int withhold_tile, cudaStream_t stream, int* n_launches);
+
+// The dense kernel's launcher (fwd_sm100_dense.cu).
+cudaError_t launch_dense(const Problem& p, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
+                         __nv_bfloat16* out, const WsPtrs& ws, int32_t* counts, uint32_t* mask_out, int sms,
+                         long long wait_limit, int withhold_tile, cudaStream_t stream, int* n_launches);
 
 }  // namespace fwd
 }  // namespace sol
