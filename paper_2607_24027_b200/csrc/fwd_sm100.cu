@@ -188,12 +188,9 @@ __device__ void router_role(Shared<C>& sm, const Params& p, int lane) {
   PROF_DECL
   if (lane == 0) CTATRACE(0, prof::gtimer());
   while (alive) {
-    // the first work item is the CTA's own number (a round trip to memory less at the start), then the counter's
-    int w = (int)blockIdx.x;
-    if (n_item > 0) {
-      if (lane == 0) w = (int)gridDim.x + atomicAdd(p.status + kStatusTileCounter, 1);
-      w = __shfl_sync(full, w, 0);
-    }
+    int w = 0;
+    if (lane == 0) w = atomicAdd(p.status + kStatusTileCounter, 1);
+    w = __shfl_sync(full, w, 0);
     if (w >= p.total_work) break;
     if (lane == 0) ITRACE(n_item, 0);
     const int bh = w / p.Nq, i = w - bh * p.Nq;
