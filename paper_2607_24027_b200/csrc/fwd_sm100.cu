@@ -721,8 +721,7 @@ __device__ void softmax_role(Shared<C>& sm, const Params& p, uint32_t tmem, int 
           const float2 t = __fadd2_rn(s_a, s_b);
           l += t.x + t.y;
         }
-        if constexpr (kHalf == 64) tmem_st_32x32b_x32(t_s, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
-        else tmem_st_32x32b_x16(t_s, *reinterpret_cast<uint32_t(*)[16]>(&sr[0]));
+        tmem_st_32x32b_x32(t_s, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
       }
       PROF_ADD(8)                                                                      // prof 8: load + arithmetic
       tmem_st_wait();
