@@ -360,6 +360,18 @@ __device__ void producer_role(Shared<C>& sm, const Params& p, unsigned char* sQ,
   using TBytes = std::integral_constant<int, C::kTileBytes>;
   using TBox = std::integral_constant<int, C::kBoxBytes>;
   auto release = [&](uint32_t r) { mbar_arrive(&sm.rec_empty[r]); };
+  // Where no V load is owed, the V cursor has nothing left up to the record that the K cursor is done with, and
+  // hands it back along with it: by itself it would move on only for the next V load, while the router may have to
+  // write more records without a tile (keep-or-drop mode) than the ring holds to get there.
+  auto release_k = [&](uint32_t r) {
+    release(r);
+    if (n_k != n_v) return;
+    for (; cur_v.n_rec != cur_k.n_rec; ++cur_v.n_rec) release(cur_v.n_rec % kRecords);
+    release(r);
+    ++cur_v.n_rec;
+    cur_v.rec = nullptr;
+    cur_v.e = cur_v.end = 0;
+  };
   bool k_end = false, have_k = false, ok = true;
   uint32_t dk = 0;
   for (;;) {
@@ -368,7 +380,7 @@ __device__ void producer_role(Shared<C>& sm, const Params& p, unsigned char* sQ,
       if (!have_k) {
         // never sleep on the router while a V load is owed: the router may itself be waiting for
         // the V cursor to hand a record back
-        dk = next_desc(sm, cur_k, wait_limit, PROF_ACC(0), release, n_k == n_v);      // prof 0: no record yet
+        dk = next_desc(sm, cur_k, wait_limit, PROF_ACC(0), release_k, n_k == n_v);      // prof 0: no record yet
         if (dk == kDescNone) break;
         if (dk == kDescAbort) { ok = false; break; }
         if (dk == kDescStop) { k_end = true; break; }

@@ -101,7 +101,7 @@ struct Shared {
   uint64_t k_full[kStages], k_empty[kStages], v_full[kStages], v_empty[kStages];
   // one of each per stream:
   uint64_t q_full[2], q_empty[2];
-  uint64_t o_free[2];           // the accumulator of a finished work item has been read
+  uint64_t o_free[2];           // the accumulator of a finished work item (with a tile) has been read
   // one of each per stream and score buffer:
   uint64_t s_full[2][2];        // the scores of a tile are in TMEM
   uint64_t p_full[2][2];        // its P is in TMEM
@@ -488,6 +488,7 @@ __device__ void mma_role(Shared<C>& sm, const Params& p, unsigned char* sQ, unsi
   const bool leader = elect_one();
   Cursor ck, cv;
   uint32_t n_qk = 0, n_pv = 0;                 // tiles whose Q K^T / P V has been issued
+  uint32_t n_acc = 0;                          // work items with a tile of the stream
   uint32_t started = 0;                        // query blocks of the stream whose accumulator holds something
   auto ready = [&](uint64_t* bar, uint32_t parity) { return __all_sync(full, mbar_test_wait(bar, parity)) != 0; };
   auto open = [&](Cursor& c) {                 // the next record, which is there
@@ -580,13 +581,8 @@ __device__ void mma_role(Shared<C>& sm, const Params& p, unsigned char* sQ, unsi
       //  stream the V side may be done first, and must not run on into a record that is not written yet)
       if ((int)(ck.n_rec - cv.n_rec) > 0 || (cv.n_rec == ck.n_rec && ck.rec)) { open(cv); moved = true; }
     } else if (cv.e == cv.n) {
-      // (an item without any tile still answers for the previous one's accumulator)
-      const bool empty = cv.exists && cv.last_chunk && cv.last < 0 && cv.fresh;
-      if (!empty || cv.n_item < 2 || ready(&sm.o_free[s], (cv.n_item - 2) & 1)) {
-        if (empty) cv.fresh = false;
-        close(cv);
-        moved = true;
-      }
+      close(cv);
+      moved = true;
     } else if (!cv.use) {
       if (ready(&sm.v_full[cv.slot], cv.par)) {
         if (leader) mbar_arrive(&sm.v_empty[cv.slot]);
@@ -596,9 +592,9 @@ __device__ void mma_role(Shared<C>& sm, const Params& p, unsigned char* sQ, unsi
     } else if (n_pv != n_qk) {
       bool go = ready(&sm.v_full[cv.slot], cv.par);
       if (go && cv.fresh) {
-        // the first P V of a work item overwrites O: the previous item's epilogue must have read it
-        go = cv.n_item < 2 || ready(&sm.o_free[s], (cv.n_item - 2) & 1);
-        if (go) { cv.fresh = false; started = 0; }
+        // the first P V of a work item overwrites O: the epilogue of the last item with a tile must have read it
+        go = n_acc == 0 || ready(&sm.o_free[s], (n_acc - 1) & 1);
+        if (go) { cv.fresh = false; started = 0; ++n_acc; }
       }
       const uint32_t x = n_pv & 1;
       if (go) {
@@ -824,7 +820,7 @@ __device__ void softmax_role(Shared<C>& sm, const Params& p, uint32_t tmem, int 
           // the accumulator is in registers: the next item's first P V may overwrite it
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(&sm.o_free[s]);
+          if (lane == 0 && g != g_item0) mbar_arrive(&sm.o_free[s]);   // (nothing waits for an item without tiles)
         }
         if (store) {
 #pragma unroll
