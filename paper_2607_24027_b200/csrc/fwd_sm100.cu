@@ -334,7 +334,9 @@ __device__ void router_role(Shared<C>& sm, const Params& p, int lane) {
 // ahead of the V loads: that is the order in which the slots come free (a K slot when its score
 // GEMM retires, a V slot a softmax pass and a P V later), so an in-order thread seldom waits for a
 // slot while another load could go.
-template <class C>
+//
+// kEmptyChunks: a record may hold no tile (keep-or-drop mode; otherwise every chunk has its approximate tile or routed ones).
+template <class C, bool kEmptyChunks>
 __device__ void producer_role(Shared<C>& sm, const Params& p, unsigned char* sQ, unsigned char* sKV,
                               const CUtensorMap* tm_q, const CUtensorMap* tm_k, const CUtensorMap* tm_v,
                               const CUtensorMap* tm_kc, const CUtensorMap* tm_vm) {
@@ -360,27 +362,33 @@ __device__ void producer_role(Shared<C>& sm, const Params& p, unsigned char* sQ,
   using TBytes = std::integral_constant<int, C::kTileBytes>;
   using TBox = std::integral_constant<int, C::kBoxBytes>;
   auto release = [&](uint32_t r) { mbar_arrive(&sm.rec_empty[r]); };
-  // Where no V load is owed, the V cursor has nothing left up to the record that the K cursor is done with, and
-  // hands it back along with it: by itself it would move on only for the next V load, while the router may have to
-  // write more records without a tile (keep-or-drop mode) than the ring holds to get there.
-  auto release_k = [&](uint32_t r) {
-    release(r);
-    if (n_k != n_v) return;
-    for (; cur_v.n_rec != cur_k.n_rec; ++cur_v.n_rec) release(cur_v.n_rec % kRecords);
-    release(r);
-    ++cur_v.n_rec;
-    cur_v.rec = nullptr;
-    cur_v.e = cur_v.end = 0;
-  };
   bool k_end = false, have_k = false, ok = true;
   uint32_t dk = 0;
+  auto next_k = [&](bool block) {
+    if constexpr (!kEmptyChunks) {
+      return next_desc(sm, cur_k, wait_limit, PROF_ACC(0), release, block);           // prof 0: no record yet
+    } else {
+      // Where no V load is owed, the V cursor has nothing left up to the record that the K cursor is done with, and
+      // hands it back along with it: by itself it would move on only for the next V load, while the router may have
+      // to write more records without a tile than the ring holds to get there.
+      return next_desc(sm, cur_k, wait_limit, PROF_ACC(0), [&](uint32_t r) {
+        release(r);
+        if (n_k != n_v) return;
+        for (; cur_v.n_rec != cur_k.n_rec; ++cur_v.n_rec) release(cur_v.n_rec % kRecords);
+        release(r);
+        ++cur_v.n_rec;
+        cur_v.rec = nullptr;
+        cur_v.e = cur_v.end = 0;
+      }, block);
+    }
+  };
   for (;;) {
     // K side (and Q): up to kLead tiles ahead of the V side
     while (!k_end && (int)(n_k - n_v) < kLead) {
       if (!have_k) {
         // never sleep on the router while a V load is owed: the router may itself be waiting for
         // the V cursor to hand a record back
-        dk = next_desc(sm, cur_k, wait_limit, PROF_ACC(0), release_k, n_k == n_v);      // prof 0: no record yet
+        dk = next_k(n_k == n_v);
         if (dk == kDescNone) break;
         if (dk == kDescAbort) { ok = false; break; }
         if (dk == kDescStop) { k_end = true; break; }
@@ -827,7 +835,7 @@ __device__ void softmax_role(Shared<C>& sm, const Params& p, uint32_t tmem, int 
   if (lane == 0 && warp_in_group == 0 && h == 0) { PROF_FLUSH(3); CTATRACE(3, prof::gtimer()); }
 }
 
-template <class C, bool kFromMask>
+template <class C, bool kFromMask, bool kEmptyChunks>
 __global__ void __launch_bounds__(kThreads, 1)
 fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_kc,
@@ -873,7 +881,7 @@ fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   } else if (warp == kWarpRouter) {
     router_role<C, kFromMask>(sm, p, lane);
   } else if (warp == kWarpProducer) {
-    if (lane == 0) producer_role<C>(sm, p, sQ, sKV, &tm_q, &tm_k, &tm_v, &tm_kc, &tm_vm);
+    if (lane == 0) producer_role<C, kEmptyChunks>(sm, p, sQ, sKV, &tm_q, &tm_k, &tm_v, &tm_kc, &tm_vm);
   } else if (warp == kWarpQK) {
     mma_qk_role<C>(sm, p, sQ, sKV, tmem);
   } else {
@@ -891,9 +899,11 @@ int g_withhold_tile = -1;
 template <class C>
 cudaError_t launch_instance(const Problem& p, const Maps& m, const Params& prm, int grid, cudaStream_t stream) {
   const size_t smem = 1024 + C::kQBytes + (kKStages + kVStages) * C::kTileBytes + sizeof(Shared<C>);
-  // the pre-pass variant is a kernel of its own, so that the in-kernel router's code is what it is without it
-  auto kernel = p.routing == SOL_ROUTING_PREPASS && p.mode != SOL_MODE_DENSE ? fwd_sm100_kernel<C, true>
-                                                                            : fwd_sm100_kernel<C, false>;
+  // The variants are kernels of their own, so that each has no code of the others in it: where the hot loop's neighbours
+  // change, its pace does (the keep-or-drop handling in the default kernel: 18.3 against 18.0 ms at 40 heads x 75 600 tokens).
+  const bool mask = p.routing == SOL_ROUTING_PREPASS && p.mode != SOL_MODE_DENSE;
+  auto kernel = p.mode == SOL_MODE_EXACT_ONLY ? (mask ? fwd_sm100_kernel<C, true, true> : fwd_sm100_kernel<C, false, true>)
+                                              : (mask ? fwd_sm100_kernel<C, true, false> : fwd_sm100_kernel<C, false, false>);
   return launch_after(kernel, dim3(grid), kThreads, smem, 0, stream, m.q, m.k, m.v, m.kc, m.vm, prm);
 }
 
