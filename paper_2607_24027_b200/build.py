@@ -17,7 +17,8 @@ LIB = os.path.join(PKG, "libsol_attn.so")
 SOURCES = ["api.cu", "pool.cu", "fwd_mma_sync.cu", "fwd_sm100.cu", "fwd_sm100_b64.cu", "fwd_sm100_dense.cu",
            "thresholds_static.cu", "route_materialized.cu", "route_prepass.cu"]
 HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "ptx_sm100.cuh"), os.path.join(CSRC, "tmap.cuh"),
-           os.path.join(CSRC, "fwd_sm100_common.cuh"), os.path.join(CSRC, "proxy_tile.cuh"),
+           os.path.join(CSRC, "fwd_sm100_common.cuh"), os.path.join(CSRC, "fwd_sm100_records.cuh"),
+           os.path.join(CSRC, "proxy_tile.cuh"),
            os.path.join(CSRC, "fwd_sm100_prof.cuh"),
            os.path.join(ROOT, "include", "sol_attn.h")]
 
