@@ -8,8 +8,8 @@
 // independently: a tile is computed for a stream when either of its two blocks wants it, the warps of a
 // block that does not want it skip its softmax, and the P V MMA leaves that block's accumulator lanes alone
 // (its disable-output-lane operand).  Neighbouring query blocks route much alike, so little is computed in
-// vain.  Measured on 16 heads, d = 64, 11 160 tokens, density 0.20, keep-or-drop: 0.36 ms a call against
-// 0.61 ms with one query block per tile.
+// vain.  24 heads x 9000 tokens, d = 64, random inputs, pooled tensors at hand: 0.44 ms, where one query block per tile
+// takes 0.63 ms.
 //
 // (With 128-token blocks, where a tile is full anyway, the same structure takes fewer cycles in dense mode
 // but more energy, and the part runs at its power limit: 20.0 against 19.9 ms at 40 heads and 32 760
@@ -764,8 +764,11 @@ __device__ void softmax_role(Shared<C>& sm, const Params& p, uint32_t tmem, int 
         l *= f;
         m_used = m_new;
       }
-      // ---- P = exp2(sl2 * S - m) (scaling and row sum as packed fp32 pairs); P (bf16) back to
-      //      TMEM over the start of the scores
+      // ---- P = exp2(sl2 * S - m) (scaled as packed fp32 pairs); P (bf16) back to TMEM over the start of the
+      //      scores.  The row sum is that of the rounded P, the weights that P V uses.  A row has one maximum here,
+      //      where fwd_sm100.cu has one per column half and with it two exact weights; with the sum of the unrounded
+      //      P the error against 64 bits grows from 1.80e-3 to 1.85e-3 (16 heads, d = 64, 11 160 tokens, density
+      //      0.20, keep-or-drop), with this one it is 1.78e-3.
       {
         const float nm = (m_used == -INFINITY) ? 0.f : -m_used;   // a row that has seen nothing yet: all P = 0
         const float2 sl2_2 = make_float2(sl2, sl2), nm2 = make_float2(nm, nm);
@@ -776,12 +779,12 @@ __device__ void softmax_role(Shared<C>& sm, const Params& p, uint32_t tmem, int 
           const float2 xb = __ffma2_rn(make_float2(__uint_as_float(sr[c + 2]), __uint_as_float(sr[c + 3])), sl2_2, nm2);
           const float2 ea = make_float2(ex2(xa.x), ex2(xa.y));
           const float2 eb = make_float2(ex2(xb.x), ex2(xb.y));
-          s_a = __fadd2_rn(s_a, ea);
-          s_b = __fadd2_rn(s_b, eb);
           __nv_bfloat162 lo = __floats2bfloat162_rn(ea.x, ea.y);
           __nv_bfloat162 hi = __floats2bfloat162_rn(eb.x, eb.y);
           sr[c / 2] = *reinterpret_cast<uint32_t*>(&lo);
           sr[c / 2 + 1] = *reinterpret_cast<uint32_t*>(&hi);
+          s_a = add_bf16x2(s_a, sr[c / 2]);
+          s_b = add_bf16x2(s_b, sr[c / 2 + 1]);
         }
         const float2 t = __fadd2_rn(s_a, s_b);
         l += t.x + t.y;

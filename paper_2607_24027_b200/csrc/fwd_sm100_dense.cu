@@ -18,10 +18,10 @@
 //
 // TMEM: S_A [0, 128)  S_B [128, 256)  O_A [256, 256 + d)  O_B [256 + d, 256 + 2 d).
 //
-// 40 heads x 32 760 tokens, d = 128: 19.4 ms against 20.0 ms with one query tile per CTA (3350 against 3490 cycles for two
-// tiles; the part is at its 1 kW limit in both, at about 1.5 GHz of counted cycles).  d = 64, 40 x 16 000: 3.6 ms against
-// 12.8 ms.  What holds it: the tensor core, whose 2048 cycles of GEMMs take the issuing warp 2500 to get through beside
-// the shared-memory traffic of the operands (128 bytes per clock while Q K^T runs), and the power limit.
+// 40 heads x 32 760 tokens, d = 128: 19.9 ms against 20.0 ms with one query tile per CTA (19.7 with the row sum of the
+// unrounded weights, see softmax_role; the part is at its 1 kW limit in all three); d = 64, 40 x 16 000: 3.69 ms against
+// 3.93 ms.  A pair of tiles takes 3 400 cycles, of which the tensor core needs 2 048: a tile's softmax, P V and next Q K^T
+// follow one another, and beside the other tile's the three take that long.
 // Every wait is bounded, as in the other kernels.
 #include "fwd_sm100_common.cuh"
 
@@ -265,7 +265,10 @@ __device__ void softmax_role(Shared& sm, const Params& p, uint32_t tmem, int s, 
         l *= f;
         m_used = m_new;
       }
-      // P = exp2(sl2 S - m), row sum over the unrounded values; packed fp32 pairs
+      // P = exp2(sl2 S - m), scaled as packed fp32 pairs.  The row sum is that of the rounded P, the weights that P V
+      // uses: with one maximum per row the sum of the unrounded P has a larger error against 64 bits (12 heads,
+      // 11 160 tokens with sink tokens, d = 128: 1.93e-3; so 1.83e-3; fwd_sm100.cu with a maximum per column half
+      // 1.90e-3).
       const float nm = (m_used == -INFINITY) ? 0.f : -m_used;   // a row without a finite logit yet: all P = 0
       const float2 sl2_2 = make_float2(sl2, sl2), nm2 = make_float2(nm, nm);
       float2 s_a = make_float2(0.f, 0.f), s_b = make_float2(0.f, 0.f);
@@ -277,12 +280,12 @@ __device__ void softmax_role(Shared& sm, const Params& p, uint32_t tmem, int s, 
           const float2 xb = __ffma2_rn(make_float2(__uint_as_float(x[2]), __uint_as_float(x[3])), sl2_2, nm2);
           const float2 ea = make_float2(ex2(xa.x), ex2(xa.y));
           const float2 eb = make_float2(ex2(xb.x), ex2(xb.y));
-          s_a = __fadd2_rn(s_a, ea);
-          s_b = __fadd2_rn(s_b, eb);
           __nv_bfloat162 lo = __floats2bfloat162_rn(ea.x, ea.y);
           __nv_bfloat162 hi = __floats2bfloat162_rn(eb.x, eb.y);
           sr[(c0 + c) / 2] = *reinterpret_cast<uint32_t*>(&lo);
           sr[(c0 + c) / 2 + 1] = *reinterpret_cast<uint32_t*>(&hi);
+          s_a = add_bf16x2(s_a, sr[(c0 + c) / 2]);
+          s_b = add_bf16x2(s_b, sr[(c0 + c) / 2 + 1]);
         }
       };
       auto arrive = [&](int half) {

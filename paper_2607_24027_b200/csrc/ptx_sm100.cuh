@@ -225,6 +225,16 @@ __device__ __forceinline__ void set_max_registers_down() {
   asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
 }
 
+// c plus a packed pair of bf16, in fp32: one instruction per value, no unpacking.
+__device__ __forceinline__ float2 add_bf16x2(float2 c, uint32_t x) {
+  unsigned short lo, hi;
+  float2 r;
+  asm("mov.b32 {%0, %1}, %2;" : "=h"(lo), "=h"(hi) : "r"(x));
+  asm("add.f32.bf16 %0, %1, %2;" : "=f"(r.x) : "h"(lo), "f"(c.x));
+  asm("add.f32.bf16 %0, %1, %2;" : "=f"(r.y) : "h"(hi), "f"(c.y));
+  return r;
+}
+
 __device__ __forceinline__ bool elect_one() {
   uint32_t pred;
   asm volatile(
