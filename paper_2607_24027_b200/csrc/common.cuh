@@ -43,6 +43,23 @@ struct Problem {
   int routing;             // SOL_ROUTING_*: where the comparison of Eq. (4) is evaluated
 };
 
+// Dense mode does not depend on the block size: two query tiles of 128 rows per CTA (fwd_sm100_dense.cu), or the kernel for
+// the block size?  All tiles cost the same, so a call is done in rounds of one tile per SM, or of one pair of tiles.
+//   128-token blocks (fwd_sm100.cu, one tile): a pair takes as long as 1.97 single tiles at d = 128 and 1.78 at d = 64.
+//     d = 128, us with single tiles / pairs: 2 x 4096 tokens (rounds 1 / 1) 39 / 68; 24 x 1024 (2 / 1) 28.3 / 24.6;
+//     24 x 2048 (3 / 2) 60 / 73; 24 x 4096 (6 / 3) 227 / 222; 30 x 4096 (7 / 4) 269 / 282; 12 x 11 160 (8 / 4) 773 / 744;
+//     24 x 8500 (11 / 6) 869 / 890; 40 x 8192 (18 / 9) 1341 / 1304.
+//     d = 64: 12 x 4096 (3 / 2) 101 / 115; 24 x 4096 (6 / 3) 188 / 169; 30 x 4096 (7 / 4) 221 / 221; 40 x 16 000 (34 / 18)
+//     3918 / 3695.
+//   64-token blocks (fwd_sm100_b64.cu): that kernel also takes 256 rows at a time, but tiles of 64 keys; pairs take 0.74 to
+//     1.00 of its time from 1 x 128 to 40 x 16 000 tokens.
+inline bool dense_in_pairs(int BH, int N, int d, int block_k, int sms) {
+  if (block_k == 64) return true;
+  const long long tiles = (long long)BH * ceil_div(N, 128), pairs = (long long)BH * ceil_div(N, 256);
+  const long long rounds = (tiles + sms - 1) / sms, pair_rounds = (pairs + sms - 1) / sms;
+  return (d == 128 ? 197 : 178) * pair_rounds <= 100 * rounds;
+}
+
 // Byte offsets into the workspace (all multiples of 1024).
 struct WsLayout {
   size_t status;  // int32[kStatusWords]

@@ -681,15 +681,7 @@ cudaError_t launch_fwd_sm100(const Problem& p, const __nv_bfloat16* q, const __n
   int sms = 0;
   cudaError_t e = fwd::sm_count(&sms);
   if (e != cudaSuccess) return e;
-  // Dense mode does not depend on the block size; all tiles cost the same, so it is done in rounds of one tile
-  // (this kernel) or one pair of tiles (the dense one) per SM, and a pair takes 0.97 of two single tiles (20.0 against
-  // 19.4 ms at 40 heads x 32 760 tokens, d = 128; 24 x 8500: 0.838 against 0.847 ms, 11 rounds against 6; 48 x 700: 0.027
-  // against 0.021 ms, 2 against 1).  With d = 64 or 64-token blocks the alternative computes tiles of 64 keys: 40 x 16 000,
-  // d = 64: 4.5 against 3.6 ms.
-  const long long tiles = (long long)p.BH * ceil_div(p.N, fwd::kRowsQ), pairs = (long long)p.BH * ceil_div(p.N, 2 * fwd::kRowsQ);
-  const long long rounds = (tiles + sms - 1) / sms, pair_rounds = (pairs + sms - 1) / sms;
-  const bool whole_tiles = p.d == 128 && p.block_k == 128;
-  if (p.mode == SOL_MODE_DENSE && (whole_tiles ? 200 * pair_rounds <= 206 * rounds : rounds > 1))
+  if (p.mode == SOL_MODE_DENSE && dense_in_pairs(p.BH, p.N, p.d, p.block_k, sms))
     return fwd::launch_dense(p, q, k, v, out, ws, counts, mask_out, sms, fwd::g_wait_limit, fwd::g_withhold_tile, stream,
                              n_launches);
   if (p.block_k == 64)
