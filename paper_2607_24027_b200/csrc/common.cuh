@@ -51,10 +51,11 @@ struct Problem {
 //     24 x 8500 (11 / 6) 869 / 890; 40 x 8192 (18 / 9) 1341 / 1304.
 //     d = 64: 12 x 4096 (3 / 2) 101 / 115; 24 x 4096 (6 / 3) 188 / 169; 30 x 4096 (7 / 4) 221 / 221; 40 x 16 000 (34 / 18)
 //     3918 / 3695.
-//   64-token blocks (fwd_sm100_b64.cu): that kernel also takes 256 rows at a time, but tiles of 64 keys; pairs take 0.74 to
-//     1.00 of its time from 1 x 128 to 40 x 16 000 tokens.
+//   64-token blocks: up to one block per SM fwd_sm100.cu (2 x 4096 tokens, d = 128: 55 / 68).  Above that the other kernel,
+//     fwd_sm100_b64.cu, also takes 256 rows at a time, but tiles of 64 keys; pairs take 0.74 to 0.85 of its time up to
+//     40 x 16 000 tokens.
 inline bool dense_in_pairs(int BH, int N, int d, int block_k, int sms) {
-  if (block_k == 64) return true;
+  if (block_k == 64) return (long long)BH * ceil_div(N, 64) > sms;
   const long long tiles = (long long)BH * ceil_div(N, 128), pairs = (long long)BH * ceil_div(N, 256);
   const long long rounds = (tiles + sms - 1) / sms, pair_rounds = (pairs + sms - 1) / sms;
   return (d == 128 ? 197 : 178) * pair_rounds <= 100 * rounds;

@@ -1,8 +1,8 @@
 // Sol-Attn fused forward (Algorithm 1) for sm_100a: TMA + tcgen05.mma + TMEM.
 //
-// Persistent kernel for 128-token blocks, one CTA of 384 threads per SM, compiled for d in {64, 128}
-// (fwd_sm100_b64.cu is the one for 64-token blocks).  A CTA owns one query block at a time and is split
-// into warp roles that talk through mbarriers:
+// Persistent kernel, one CTA of 384 threads per SM, compiled for d in {64, 128} and blocks of 128 or 64 tokens (64: for
+// calls of at most one query block per SM; fwd_sm100_b64.cu takes the others).  A CTA owns one query block at a time and is
+// split into warp roles that talk through mbarriers:
 //
 //   router   (warp 8)  pulls (head, query block) work items from a global counter and walks the
 //                      pooled keys in chunks of `block` blocks.  For every block it evaluates the
@@ -25,6 +25,9 @@
 //                      denominator, mean value times n_j in the numerator) or -inf for routed /
 //                      padded columns.  O_h is rescaled lazily, only when the running maximum
 //                      grows by more than 2^8.
+//
+// The query tile of the MMAs always has 128 rows (the M of a one-CTA tcgen05.mma at full rate); with 64-token
+// blocks its upper 64 rows belong to the next query block, take part in the arithmetic and are never stored.
 //
 // TMEM (512 columns): S0 [0, block)  S1 [block, 2 block)  O0 [256, 256 + d)  O1 [256 + d, 256 + 2 d);
 // P_h (bf16) of a tile overwrites the start of group h's half of that tile's S buffer.
@@ -499,7 +502,8 @@ __device__ void softmax_role(Shared<C>& sm, const Params& p, uint32_t tmem, int 
           const float2 t = __fadd2_rn(s_a, s_b);
           l += t.x + t.y;
         }
-        tmem_st_32x32b_x32(t_s, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
+        if constexpr (kHalf == 64) tmem_st_32x32b_x32(t_s, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
+        else tmem_st_32x32b_x16(t_s, *reinterpret_cast<uint32_t(*)[16]>(&sr[0]));
       }
       PROF_ADD(8)                                                                      // prof 8: load + arithmetic
       tmem_st_wait();
@@ -684,7 +688,10 @@ cudaError_t launch_fwd_sm100(const Problem& p, const __nv_bfloat16* q, const __n
   if (p.mode == SOL_MODE_DENSE && dense_in_pairs(p.BH, p.N, p.d, p.block_k, sms))
     return fwd::launch_dense(p, q, k, v, out, ws, counts, mask_out, sms, fwd::g_wait_limit, fwd::g_withhold_tile, stream,
                              n_launches);
-  if (p.block_k == 64)
+  // 64-token blocks: several query blocks per CTA need more blocks than SMs.  Up to one block per SM a CTA has one in either
+  // kernel, and here both softmax warpgroups share its columns.  Pooled tensors at hand, us here / there: 2 heads x 1024
+  // tokens, d = 64 14.3 / 16.4; 2 x 4096, d = 64 26.2 / 32.8, d = 128 28.7 / 36.9.
+  if (p.block_k == 64 && (long long)p.BH * p.Nq > sms)
     return fwd::launch_b64(p, q, k, v, out, ws, tau, counts, mask_out, fwd::g_wait_limit, fwd::g_withhold_tile, stream,
                            n_launches);
   fwd::Maps m;
@@ -694,8 +701,12 @@ cudaError_t launch_fwd_sm100(const Problem& p, const __nv_bfloat16* q, const __n
   prm.wait_limit = fwd::g_wait_limit;
   prm.withhold_tile = fwd::g_withhold_tile;
   const int grid = prm.total_work < sms ? prm.total_work : sms;
-  e = p.d == 128 ? fwd::launch_instance<fwd::Cfg<128, 128>>(p, m, prm, grid, stream)
-                 : fwd::launch_instance<fwd::Cfg<64, 128>>(p, m, prm, grid, stream);
+  if (p.block_k == 128)
+    e = p.d == 128 ? fwd::launch_instance<fwd::Cfg<128, 128>>(p, m, prm, grid, stream)
+                   : fwd::launch_instance<fwd::Cfg<64, 128>>(p, m, prm, grid, stream);
+  else
+    e = p.d == 128 ? fwd::launch_instance<fwd::Cfg<128, 64>>(p, m, prm, grid, stream)
+                   : fwd::launch_instance<fwd::Cfg<64, 64>>(p, m, prm, grid, stream);
   if (n_launches) *n_launches += 1;
   return e;
 }

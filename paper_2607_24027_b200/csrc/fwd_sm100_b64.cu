@@ -36,9 +36,9 @@
 //                      -inf for routed / padded columns.  O is rescaled lazily, only when the running
 //                      maximum grows by more than 2^8.
 //
-// Work item size: four query blocks share loads and tiles best, but a problem with fewer blocks than SMs is
-// cut into items of one block, and one with fewer than two per SM into items of two (a stream each), so that
-// every SM has something to do.
+// Work item size: four query blocks share loads and tiles best, but a problem with fewer than two blocks per SM is cut into
+// items of two (a stream each), so that every SM has something to do.  (One with at most one block per SM goes to
+// fwd_sm100.cu.)
 //
 // TMEM (512 columns): stream s, score buffer x: S at 64 (2 s + x); O_s at 256 + s d.  P (bf16) of a tile
 // overwrites the start of its S.
@@ -232,7 +232,6 @@ __device__ void router_role(Shared<C>& sm, const Params& p, int lane) {
               const float4 kk = row[piece];
 #pragma unroll
               for (int u = 0; u < kNQ; ++u) {
-                if (u > 0 && p.per_item == 1) break;          // items of one block, where latency is all
                 const float4 qq = qv[u * (kD / 4) + piece];
                 a0[u] = fmaf(qq.x, kk.x, a0[u]);
                 a1[u] = fmaf(qq.y, kk.y, a1[u]);
@@ -935,7 +934,7 @@ cudaError_t launch_b64(const Problem& p, const __nv_bfloat16* q, const __nv_bflo
   if (e != cudaSuccess) return e;
   // as many query blocks per work item as still leave every SM one
   const long long blocks = (long long)p.BH * p.Nq;
-  prm.per_item = blocks <= sms ? 1 : (blocks <= 2LL * sms ? 2 : kNQ);
+  prm.per_item = blocks <= 2LL * sms ? 2 : kNQ;
   prm.items_per_head = ceil_div(p.Nq, prm.per_item);
   prm.total_work = p.BH * prm.items_per_head;
   const int grid = prm.total_work < sms ? prm.total_work : sms;

@@ -1,4 +1,5 @@
-// The routing records of the 128-token kernel, how its roles walk them, and the role that loads what they ask for.
+// The routing records of the kernel with one query block per CTA, how its roles walk them, and the role that loads what
+// they ask for.
 //
 // Included by fwd_sm100.cu behind fwd_sm100_common.cuh and its WAIT / PROF macros, and nothing here needs a GPU to
 // run: tests/record_ring.cpp compiles it for the host, with mbarriers and TMA loads of its own, and steps the roles
@@ -29,7 +30,7 @@ struct Cfg {
   static constexpr int kQBoxBytes = kRowsQ * 128;  // one box of the query tile (64 channels x 128 rows)
   static constexpr int kBoxBytes = BLK * 128;      // one box of a K-like / V-like tile
   static_assert(D == 64 || D == 128, "head dimension");
-  static_assert(BLK == kRowsQ, "a query block fills the query tile");
+  static_assert(BLK == 64 || BLK == 128, "block size");
 };
 
 // The router turns every chunk of `block` key blocks into a record: a flat list of tile descriptors

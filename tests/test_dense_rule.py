@@ -42,4 +42,4 @@ def rule(tmp_path_factory):
 def test_pairs_or_single_tiles(rule, H, N, d128, d64):
     assert rule(H, N, 128, 128) == d128
     assert rule(H, N, 64, 128) == d64
-    assert rule(H, N, 64, 64) and rule(H, N, 128, 64)
+    assert rule(H, N, 64, 64) == rule(H, N, 128, 64) == (H * -(-N // 64) > 148)

@@ -1,4 +1,4 @@
-"""The 64-token-block tcgen05 kernel: work items of one, two and four query blocks, ragged ends, every mode."""
+"""64-token blocks: the kernel with one query block per CTA, work items of two and four of them, ragged ends, every mode."""
 import numpy as np
 import pytest
 import torch
@@ -10,7 +10,7 @@ from tests.test_gpu_parity import _check_all_heads, _lib, _small_problem  # noqa
 pytestmark = pytest.mark.gpu
 
 
-# 148 SMs: up to 148 query blocks over all heads run as items of one block, up to 296 as items of two, more as items of
+# 148 SMs: up to 148 query blocks over all heads run as one block per CTA, up to 296 as items of two, more as items of
 # four; a last item that lacks one, two or three of its blocks, and last blocks of 1, 63 and 64 tokens
 @pytest.mark.parametrize("H,N,d", [(1, 64, 64), (2, 65, 128), (2, 64 * 37, 64), (20, 64 * 9 + 63, 128), (40, 64 * 8, 64),
                                    (40, 64 * 8 + 1, 128), (36, 64 * 9 + 63, 64), (30, 64 * 11, 128)])
