@@ -132,12 +132,15 @@ inline WsPtrs make_ptrs(void* base, const WsLayout& w) {
 __device__ __forceinline__ void kernel_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void kernel_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// `smem`: dynamic shared memory of this launch; `smem_most`: of any launch of the kernel.  The limit is state of the function,
+// which other host threads may be launching too, so it never follows a call's own size.
 template <class... P, class... A>
-cudaError_t launch_after(void (*kernel)(P...), dim3 grid, int threads, size_t smem, int cluster, cudaStream_t stream,
-                         A... args) {
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, int threads, size_t smem, size_t smem_most, int cluster,
+                         cudaStream_t stream, A... args) {
   cudaError_t e = cudaSuccess;
   // (48 KB is the default limit for static and dynamic shared memory together)
-  if (smem > 32 * 1024) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem_most > 32 * 1024)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_most);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;

@@ -662,7 +662,7 @@ cudaError_t launch_instance(const Problem& p, const Maps& m, const Params& prm, 
   const size_t smem = 1024 + C::kQBytes + (kKStages + kVStages) * C::kTileBytes + sizeof(Shared<C>);
   // the pre-pass variant is a kernel of its own, so that the in-kernel router's code is what it is without it
   auto kernel = p.routing == SOL_ROUTING_PREPASS && p.mode != SOL_MODE_DENSE ? fwd_sm100_kernel<C, true> : fwd_sm100_kernel<C, false>;
-  return launch_after(kernel, dim3(grid), kThreads, smem, 0, stream, m.q, m.k, m.v, m.kc, m.vm, prm);
+  return launch_after(kernel, dim3(grid), kThreads, smem, smem, 0, stream, m.q, m.k, m.v, m.kc, m.vm, prm);
 }
 
 }  // namespace

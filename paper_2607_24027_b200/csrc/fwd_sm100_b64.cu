@@ -916,7 +916,7 @@ cudaError_t launch_instance(const Problem& p, const Maps& m, const Params& prm, 
   const size_t smem = 1024 + 2 * C::kQBytes + 2 * kStages * C::kTileBytes + sizeof(Shared<C>);
   auto kernel = p.routing == SOL_ROUTING_PREPASS && p.mode != SOL_MODE_DENSE ? fwd_sm100_b64_kernel<C, true>
                                                                             : fwd_sm100_b64_kernel<C, false>;
-  return launch_after(kernel, dim3(grid), kThreads, smem, 0, stream, m.q, m.k, m.v, m.kc, m.vm, prm);
+  return launch_after(kernel, dim3(grid), kThreads, smem, smem, 0, stream, m.q, m.k, m.v, m.kc, m.vm, prm);
 }
 
 }  // namespace

@@ -414,7 +414,7 @@ fwd_sm100_dense_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
 template <int D>
 cudaError_t launch_instance(const Problem& p, const Maps& m, const Params& prm, int grid, cudaStream_t stream) {
   const size_t smem = 1024 + (2 + kSlots) * Cfg<D>::kTileBytes + sizeof(Shared);
-  return launch_after(fwd_sm100_dense_kernel<D>, dim3(grid), kThreads, smem, 0, stream, m.q, m.k, m.v, prm, p.block_q);
+  return launch_after(fwd_sm100_dense_kernel<D>, dim3(grid), kThreads, smem, smem, 0, stream, m.q, m.k, m.v, prm, p.block_q);
 }
 
 }  // namespace

@@ -508,8 +508,8 @@ static cudaError_t thresholds_impl(const Problem& p, const WsPtrs& ws, cudaStrea
   if (p.Nk <= kSmallKeys) {
     if (n_launches) *n_launches += 1;
     return launch_after(diag ? thresholds_small_kernel<D, true> : thresholds_small_kernel<D, false>,
-                        dim3(ceil_div(p.Nq, kSmallRows), p.BH), 256, sizeof(float) * p.Nk * (D + 4), 0, stream, ws, p.Nq,
-                        p.Nk, p.scale, p.beta);
+                        dim3(ceil_div(p.Nq, kSmallRows), p.BH), 256, sizeof(float) * p.Nk * (D + 4),
+                        sizeof(float) * kSmallKeys * (D + 4), 0, stream, ws, p.Nq, p.Nk, p.scale, p.beta);
   }
   if (diag) {
     key_diag_kernel<D><<<p.BH, 4 * D, 0, stream>>>(ws, p.Nk);
@@ -527,7 +527,7 @@ static cudaError_t thresholds_impl(const Problem& p, const WsPtrs& ws, cudaStrea
   const int fit = sms * 17 / 20 / p.BH;
   const int n_cta = fit < 1 ? 1 : (fit > 8 ? 8 : fit);
   if (n_launches) *n_launches += 1;
-  return launch_after(thresholds_moments_kernel<D>, dim3(n_cta, p.BH), 256, moments_smem<D>(), n_cta, stream, ws, p.Nq, p.Nk,
+  return launch_after(thresholds_moments_kernel<D>, dim3(n_cta, p.BH), 256, moments_smem<D>(), moments_smem<D>(), n_cta, stream, ws, p.Nq, p.Nk,
                       p.scale, p.beta);
 }
 

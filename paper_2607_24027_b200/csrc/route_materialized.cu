@@ -264,7 +264,8 @@ extern "C" sol_status_t sol_attn_route_materialized(const float* qbar, const flo
     int npad = 2;
     while (npad < Nk) npad <<= 1;
     const size_t smem = (size_t)npad * 8;
-    if (cudaFuncSetAttribute(row_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    // (the limit of the longest row, not of this call's: other threads may be launching the same kernel)
+    if (cudaFuncSetAttribute(row_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxRow * 8) != cudaSuccess)
       return SOL_ERR_CUDA;
     row_select_kernel<<<dim3(Nq, BH), 256, smem, st>>>(proxy_map, Nq, Nk, npad, policy, param, order, tau, counts);
   }

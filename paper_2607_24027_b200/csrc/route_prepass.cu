@@ -59,7 +59,7 @@ cudaError_t launch_route_prepass(const Problem& p, const WsPtrs& ws, const float
                                  cudaStream_t stream, int* n_launches) {
   const dim3 grid(ceil_div(p.Nk, kProxyCols), ceil_div(p.Nq, kProxyRows), p.BH);
   if (n_launches) *n_launches += 1;
-  return launch_after(mask_prepass_kernel, grid, 256, kProxySmem, 0, stream, ws.qbar, ws.kc, tau, p.forced, mask, p.Nq, p.Nk,
+  return launch_after(mask_prepass_kernel, grid, 256, kProxySmem, kProxySmem, 0, stream, ws.qbar, ws.kc, tau, p.forced, mask, p.Nq, p.Nk,
                       p.d, p.scale);
 }
 
