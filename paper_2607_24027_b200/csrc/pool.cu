@@ -130,9 +130,9 @@ template <int D, bool kDiag>
 __global__ void __launch_bounds__(256) thresholds_small_kernel(WsPtrs ws, int Nq, int Nk, float scale, float beta) {
   constexpr int LD = D + 4;                      // rows 4 banks apart: 16-byte reads of eight rows do not collide
   constexpr int G = 256 / D;                     // threads per channel
-  extern __shared__ float smem_f[];
+  extern __shared__ __align__(16) float smem_f[];
   float* ks = smem_f;                            // [Nk][LD]
-  __shared__ float qs[kSmallRows][LD];
+  __shared__ __align__(16) float qs[kSmallRows][LD];
   __shared__ float part[G][D], mean_s[D], var_s[kDiag ? D : 1];
   const int bh = blockIdx.y, i0 = blockIdx.x * kSmallRows, tid = threadIdx.x;
   const float* kc = ws.kc + (size_t)bh * Nk * D;
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(256, 2) thresholds_moments_kernel(WsPtrs ws, i
   extern __shared__ __align__(16) float smem_f[];
   float* cov = smem_f;                           // [D][D]
   float* work = smem_f + D * D;
-  __shared__ float part[G][D], sum_s[D], mean_s[D];
+  __shared__ __align__(16) float part[G][D], sum_s[D], mean_s[D];
   const int bh = blockIdx.y, tid = threadIdx.x;
   const int ty = tid / 16, tx = tid % 16;
   const float* kc = ws.kc + (size_t)bh * Nk * D;

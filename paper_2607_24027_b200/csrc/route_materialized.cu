@@ -158,7 +158,7 @@ row_select_warp_kernel(const float* __restrict__ map, long long n_rows, int Nk, 
 __global__ void __launch_bounds__(256) row_select_kernel(const float* __restrict__ map, int Nq, int Nk, int npad,
                                                          int policy, float param, int32_t* __restrict__ order,
                                                          float* __restrict__ tau, int32_t* __restrict__ counts) {
-  extern __shared__ unsigned char smem_raw[];
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   float* val = reinterpret_cast<float*>(smem_raw);
   int* idx = reinterpret_cast<int*>(val + npad);
   __shared__ double part[256];
