@@ -23,6 +23,8 @@
 // 3.93 ms.  A pair of tiles takes 3 400 cycles, of which the tensor core needs 2 048: a tile's softmax, P V and next Q K^T
 // follow one another, and beside the other tile's the three take that long.
 // Every wait is bounded, as in the other kernels.
+#include <atomic>
+
 #include "fwd_sm100_common.cuh"
 
 namespace sol {
@@ -33,6 +35,8 @@ constexpr int kCols = 128;                       // keys per tile
 constexpr int kSlots = 5;                        // ring of K and V tiles: K0 V0 K1 V1 ...
 constexpr int kWarpMma = 8, kWarpCounts = 10;
 constexpr int kTmemS = 0, kTmemO = 256;
+constexpr int kRegsSoftmax = 200, kRegsOther = 104, kRegsLaunch = 168;   // registers per thread of the roles, and at launch
+static_assert(8 * kRegsSoftmax + 4 * kRegsOther <= 12 * kRegsLaunch, "a warpgroup would wait for registers without end");
 
 template <int D>
 struct Cfg {
@@ -395,13 +399,12 @@ fwd_sm100_dense_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const uint32_t tmem = sm.tmem_base;
   kernel_wait();
 
-  // A softmax thread holds a whole row of scores: it takes registers over from the other roles
-  // (8 x 200 + 4 x 104 per lane = 12 x 168, what the CTA was launched with).
+  // A softmax thread holds a whole row of scores: it takes registers over from the other roles.
   if (warp < 8) {
-    set_max_registers_up<200>();
+    set_max_registers_up<kRegsSoftmax>();
     softmax_role<D>(sm, p, tmem, warp / 4, warp % 4, lane);
   } else {
-    set_max_registers_down<104>();
+    set_max_registers_down<kRegsOther>();
     if (warp == kWarpMma) mma_role<D>(sm, p, sQ, sKV, tmem);
     else if (warp == kWarpProducer && lane == 0) producer_role<D>(sm, p, sQ, sKV, &tm_q, &tm_k, &tm_v);
     else if (warp == kWarpCounts) counts_role(p, block, lane);
@@ -413,6 +416,15 @@ fwd_sm100_dense_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
 
 template <int D>
 cudaError_t launch_instance(const Problem& p, const Maps& m, const Params& prm, int grid, cudaStream_t stream) {
+  // the roles share out what the launch brings, which is the compiler's choice within the launch bounds
+  static std::atomic<bool> enough{false};
+  if (!enough) {
+    cudaFuncAttributes a{};
+    const cudaError_t e = cudaFuncGetAttributes(&a, fwd_sm100_dense_kernel<D>);
+    if (e != cudaSuccess) return e;
+    if (a.numRegs < kRegsLaunch) return cudaErrorInvalidConfiguration;
+    enough = true;
+  }
   const size_t smem = 1024 + (2 + kSlots) * Cfg<D>::kTileBytes + sizeof(Shared);
   return launch_after(fwd_sm100_dense_kernel<D>, dim3(grid), kThreads, smem, smem, 0, stream, m.q, m.k, m.v, prm, p.block_q);
 }
