@@ -83,7 +83,7 @@ sol::Problem make_problem(int B, int H, int N, int d, int block_q, int block_k, 
                           int layout = SOL_LAYOUT_BHND) {
   sol::Problem p{};
   p.B = B; p.H = H; p.N = N; p.d = d; p.block_q = block_q; p.block_k = block_k;
-  p.BH = B * H;
+  p.BH = p.call_heads = B * H;
   p.Nq = sol::ceil_div(N, block_q);
   p.Nk = sol::ceil_div(N, block_k);
   p.scale = scale > 0.f ? scale : 1.0f / std::sqrt((float)d);
@@ -216,8 +216,9 @@ sol_status_t sol_attn_route_mask(int B, int H, int N, int d, int block_q, int bl
   return e == cudaSuccess ? SOL_OK : SOL_ERR_CUDA;
 }
 
-// keep_status: a later piece of one logical call must not wipe the device status of an earlier one
-static sol_status_t forward_impl(const sol_attn_args* a, bool keep_status) {
+// keep_status: a later piece of one logical call must not wipe the device status of an earlier one.
+// call_heads: (batch, head) pairs of the whole call, if this is a piece of one (else 0)
+static sol_status_t forward_impl(const sol_attn_args* a, bool keep_status, int call_heads) {
   if (!a) return SOL_ERR_INVALID_ARG;
   sol_status_t s = check_shape(a->B, a->H, a->N, a->d, a->block_q, a->block_k, true);
   if (s != SOL_OK) return s;
@@ -241,6 +242,7 @@ static sol_status_t forward_impl(const sol_attn_args* a, bool keep_status) {
   sol::Problem p = make_problem(a->B, a->H, a->N, a->d, a->block_q, a->block_k, a->threshold, a->scale, a->mode,
                                 a->estimator, a->mode == SOL_MODE_DENSE ? nullptr : a->forced_blocks, a->layout);
   p.routing = prepass ? SOL_ROUTING_PREPASS : SOL_ROUTING_FUSED;
+  if (call_heads > 0) p.call_heads = call_heads;
   int impl = a->impl;
   if (impl == SOL_IMPL_AUTO) impl = sol::fwd_sm100_supports(p) ? SOL_IMPL_TCGEN05 : SOL_IMPL_MMA_SYNC;
   if (impl == SOL_IMPL_TCGEN05 && !sol::fwd_sm100_supports(p)) return SOL_ERR_UNSUPPORTED_SHAPE;
@@ -274,7 +276,7 @@ static sol_status_t forward_impl(const sol_attn_args* a, bool keep_status) {
   return e == cudaSuccess ? SOL_OK : SOL_ERR_CUDA;
 }
 
-sol_status_t sol_attn_forward_ex(const sol_attn_args* a) { return forward_impl(a, false); }
+sol_status_t sol_attn_forward_ex(const sol_attn_args* a) { return forward_impl(a, false, 0); }
 
 sol_status_t sol_attn_forward(const void* q, const void* k, const void* v, void* out, int B, int H, int N,
                               int d, int block_q, int block_k, float threshold, sol_stream_t stream) {
@@ -344,7 +346,7 @@ sol_status_t sol_attn_forward_host(const void* hq, const void* hk, const void* h
     a.workspace = g_bound.ws; a.workspace_bytes = g_bound.bytes;
     a.counts = g_bound.counts ? g_bound.counts + (size_t)h0 * Nq : nullptr;
     a.stream = stream;
-    s = forward_impl(&a, !first);
+    s = forward_impl(&a, !first, BH);
     first = false;
     if (s != SOL_OK) return s;
     if (cudaEventRecord(hp.computed, st) != cudaSuccess || cudaStreamWaitEvent(hp.out, hp.computed, 0) != cudaSuccess ||

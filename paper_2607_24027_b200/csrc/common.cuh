@@ -34,6 +34,7 @@ struct Strides {
 struct Problem {
   int B, H, N, d, block_q, block_k;
   int BH, Nq, Nk;
+  int call_heads;    // BH of the whole call, of which this may be a group of heads: what a choice between kernels goes by
   float scale;       // logit scale
   float beta;        // standardized cutoff of Eq. (4)
   int mode;          // SOL_MODE_*

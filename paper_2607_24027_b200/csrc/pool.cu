@@ -106,6 +106,9 @@ pool_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict
   }
 }
 
+__device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+__device__ __forceinline__ float4 sub4(float4 a, float4 b) { return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w); }
+
 // mu, sigma and tau of one query block, from its raw products.
 __device__ __forceinline__ void store_threshold(const WsPtrs& ws, size_t o, float mu, float sigma, float beta) {
   ws.mu[o] = mu;
@@ -217,145 +220,203 @@ __global__ void __launch_bounds__(256) thresholds_small_kernel(WsPtrs ws, int Nq
 // (the bracket of Eq. 5 with the mu_i^2 term already folded in, which avoids the cancellation of the
 // uncentred form in fp32), then per query block mu_i = s Qbar_i . m_K, sigma_i^2 = s^2 Qbar_i C_K Qbar_i^T.
 //
-// A thread-block cluster takes one head.  Each CTA sums its share of the keys, first for the mean, then for a
-// partial C_K in registers (256 threads, 8 x 8 or 4 x 4 each); the partial sums are added through distributed
-// shared memory in rank order (bit-stable run to run), every CTA gathers the whole C_K and forms Y = Qbar C_K for
-// its share of the query blocks.  A share of up to 88 keys stays in shared memory between the two passes, and up to
-// 88 query blocks are one step: with two CTAs per SM that is the largest `work` area there is room for, and what 40
-// heads of 591 blocks give a CTA of a cluster of 7.  1.5 GFLOP at that size, 60 us; three kernels (mean on 40
-// CTAs; C_K with one shared-memory operand per FMA; quadratic form) took 198 us.
-constexpr int kMomentRows = 88;
+// A thread-block cluster takes one head.  How many CTAs it has depends on how many heads the call has, but nothing
+// that is summed does, so that a head's thresholds are the same in every call it is part of:
+//   m_K   eight slices of the keys, summed in order whichever CTA summed which;
+//   C_K   is cut by its entries, not by the keys: it is symmetric, and of its 4 x 4 blocks the ten on and above the
+//         diagonal are dealt out to the CTAs.  Every entry is the sum of four chains of FMAs, one over every fourth key
+//         (one chain over all keys, as a single CTA per head has it when the keys are dealt out, has a quarter more error).
+// Then every CTA gathers the whole C_K and forms Y = Qbar C_K for its share of the query blocks, up to 88 in one step (with
+// two CTAs per SM that is the largest `work` area there is room for).
+constexpr int kMomentRows = 88, kMeanSlices = 8;
 
 template <int D>
-constexpr size_t moments_smem() {                // C_K, then (in turn) keys / a reduced strip / pooled queries
-  constexpr size_t work = sizeof(float) * kMomentRows * D, strip = sizeof(float) * D * D / 2;
-  return sizeof(float) * D * D + (work > strip ? work : strip);
+constexpr int kMomentChunk = D == 128 ? 32 : 64; // keys in shared memory, twice
+template <int D>
+constexpr int kKeyLd = D + 16;                   // floats from one to the next: neighbours half a bank cycle apart, see below
+
+template <int D>
+constexpr size_t moments_smem() {                // C_K, then (in turn) partial sums / two chunks of keys / pooled queries
+  constexpr size_t rows = sizeof(float) * kMomentRows * D, chunks = sizeof(float) * 2 * kMomentChunk<D> * kKeyLd<D>;
+  constexpr size_t sums = sizeof(float) * kMeanSlices * 256 * 4;
+  return sizeof(float) * D * D + (rows > chunks ? (rows > sums ? rows : sums) : (chunks > sums ? chunks : sums));
 }
 
 template <int D>
 __global__ void __launch_bounds__(256, 2) thresholds_moments_kernel(WsPtrs ws, int Nq, int Nk, float scale, float beta) {
-  constexpr int T = D / 16;                      // C_K rows and columns per thread (8 or 4)
-  constexpr int G = 256 / D;
+  constexpr int T = D / 16;                      // columns of Y per thread (8 or 4)
+  constexpr int P4 = D / 4;                      // 16-byte pieces of a row
+  constexpr int E = D / 4, kBlocks = 10;         // edge of a block of C_K, blocks on and above the diagonal
+  constexpr int M = E / 4;                       // rows and columns of a block per thread (8 or 4)
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   const int n_cta = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   extern __shared__ __align__(16) float smem_f[];
   float* cov = smem_f;                           // [D][D]
   float* work = smem_f + D * D;
-  __shared__ __align__(16) float part[G][D], sum_s[D], mean_s[D];
+  __shared__ __align__(16) float sum_s[kMeanSlices][D], mean_s[D];
   const int bh = blockIdx.y, tid = threadIdx.x;
   const int ty = tid / 16, tx = tid % 16;
-  const float* kc = ws.kc + (size_t)bh * Nk * D;
-  const int per_k = ceil_div(Nk, n_cta);
-  const int j_begin = min(Nk, rank * per_k), j_end = min(Nk, j_begin + per_k);
-
-  // copies n rows of D floats to `work`
-  auto stage = [&](const float* src, int n) {
-#pragma unroll 4
-    for (int e = tid; e < n * (D / 4); e += 256)
-      reinterpret_cast<float4*>(work)[e] = reinterpret_cast<const float4*>(src)[e];
+  const int piece = tid % P4;                    // (256 is a multiple of P4: the same piece of every row it touches)
+  const float4* kc4 = reinterpret_cast<const float4*>(ws.kc + (size_t)bh * Nk * D);
+  float4* work4 = reinterpret_cast<float4*>(work);
+  auto sync = [&] {
+    if (n_cta > 1) cluster.sync();
+    else __syncthreads();
   };
   kernel_wait();
-  const bool resident = j_end - j_begin <= kMomentRows;
 
   // ---- m_K
   {
-    if (resident) {
-      stage(kc + (size_t)j_begin * D, j_end - j_begin);
-      __syncthreads();
-    }
-    const float* x = resident ? work : kc + (size_t)j_begin * D;
-    const int c = tid % D, g = tid / D;
-    float s = 0.f;
+    const int per = ceil_div(Nk, kMeanSlices);
+    for (int y = rank; y < kMeanSlices; y += n_cta) {
+      const int end = min(Nk, (y + 1) * per);
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 8
-    for (int j = g; j < j_end - j_begin; j += G) s += x[(size_t)j * D + c];
-    part[g][c] = s;
-    __syncthreads();
-    if (g == 0) {
-      float r = 0.f;
-#pragma unroll
-      for (int y = 0; y < G; ++y) r += part[y][c];
-      sum_s[c] = r;
+      for (int j = y * per + tid / P4; j < end; j += 256 / P4) x = add4(x, kc4[(size_t)j * P4 + piece]);
+      work4[y * 256 + tid] = x;
     }
-    cluster.sync();
-    if (g == 0) {
-      float other[8], r = 0.f;
+    __syncthreads();
+    for (int y = rank; y < kMeanSlices; y += n_cta)
+      if (tid < D) {
+        float r = 0.f;
 #pragma unroll
-      for (int y = 0; y < 8; ++y) other[y] = y < n_cta ? cluster.map_shared_rank(sum_s, y)[c] : 0.f;
+        for (int g = 0; g < 256 / P4; ++g) r += work[(y * 256 + g * P4) * 4 + tid];
+        sum_s[y][tid] = r;
+      }
+    sync();
+    if (tid < D) {
+      float x[kMeanSlices], r = 0.f;
 #pragma unroll
-      for (int y = 0; y < 8; ++y) r += other[y];
-      mean_s[c] = r / (float)Nk;
+      for (int y = 0; y < kMeanSlices; ++y) x[y] = cluster.map_shared_rank(&sum_s[y][0], y % n_cta)[tid];
+#pragma unroll
+      for (int y = 0; y < kMeanSlices; ++y) r += x[y];
+      mean_s[tid] = r / (float)Nk;
     }
     __syncthreads();
   }
 
-  // ---- this CTA's share of C_K.  Thread (ty, tx) owns rows and columns 4 ty + r (+ 64), 4 tx + c (+ 64).
-  float2 acc[T][T / 2];
+  // ---- this CTA's blocks of C_K, in passes over the keys of up to four blocks.  A block belongs to 64 threads, or to 128
+  //      or all 256 where a pass has fewer: 16 threads share it in patches of M x M entries, rows r0 + x (+ 16) and columns
+  //      c0 + y (+ 16), each for every fourth key, and the patches are cut into `parts` of R rows.  The two quarters of the
+  //      keys that a warp works on lie in neighbouring rows, 16 floats off in the banks: no conflicts.
+  const float4 m4 = *reinterpret_cast<const float4*>(mean_s + 4 * piece);
+  const int quarter = tid % 64 / 16, r0 = tid % 16 / 4 * 4, c0 = tid % 4 * 4;
+  constexpr int LD = kKeyLd<D>, kChunk = kMomentChunk<D>;
+  const int n_chunks = ceil_div(Nk, kChunk);
+  constexpr int kPre = kChunk * P4 / 256;        // pieces of a chunk per thread
+  float4 pre[kPre];
+  auto fetch = [&](int chunk) {
 #pragma unroll
-  for (int r = 0; r < T; ++r)
+    for (int i = 0; i < kPre; ++i) {
+      const int j = chunk * kChunk + (tid + 256 * i) / P4;
+      pre[i] = j < Nk ? kc4[(size_t)j * P4 + piece] : m4;
+    }
+  };
+  auto put = [&](int chunk) {                    // centred; keys past the last one are zero
+    float* to = work + (chunk & 1) * kChunk * LD + 4 * piece;
 #pragma unroll
-    for (int c = 0; c < T / 2; ++c) acc[r][c] = make_float2(0.f, 0.f);
-  for (int j0 = j_begin; j0 < j_end; j0 += kMomentRows) {
-    const int nj = min(kMomentRows, j_end - j0);
-    if (!resident) {
-      stage(kc + (size_t)j0 * D, nj);
+    for (int i = 0; i < kPre; ++i) *reinterpret_cast<float4*>(to + (tid + 256 * i) / P4 * LD) = sub4(pre[i], m4);
+  };
+  auto block_row = [](int b) { return (b >= 4) + (b >= 7) + (b >= 9); };
+  auto block_col = [](int b, int bi) { return b - (4 * bi - bi * (bi - 1) / 2) + bi; };
+  auto pass = [&](auto r_c, int first) {         // blocks first + slot n_cta + rank
+    constexpr int R = decltype(r_c)::value, kParts = M / R, kSlots = 4 / kParts;
+    const int group = tid / 64, part = group % kParts, b = first + group / kParts * n_cta + rank;
+    const int bi = block_row(b), bj = block_col(b, bi);
+    const int rp = r0 + part * R / 4 * 16 + part * R % 4;    // first row of the part
+    float2 acc[R][M / 2];
+#pragma unroll
+    for (int x = 0; x < R; ++x)
+#pragma unroll
+      for (int y = 0; y < M / 2; ++y) acc[x][y] = make_float2(0.f, 0.f);
+    fetch(0);
+    put(0);
+    __syncthreads();
+    for (int t = 0; t < n_chunks; ++t) {
+      if (t + 1 < n_chunks) fetch(t + 1);
+      if (b < kBlocks) {
+        const float* row = work + ((t & 1) * kChunk + quarter) * LD + bi * E + rp;
+        const float* col = work + ((t & 1) * kChunk + quarter) * LD + bj * E + c0;
+#pragma unroll 2
+        for (int j = 0; j < kChunk; j += 4) {
+          float u[R], v[M];
+          if constexpr (R >= 4) {
+#pragma unroll
+            for (int h = 0; h < R / 4; ++h)
+              *reinterpret_cast<float4*>(u + 4 * h) = *reinterpret_cast<const float4*>(row + j * LD + 16 * h);
+          } else if constexpr (R == 2) {
+            *reinterpret_cast<float2*>(u) = *reinterpret_cast<const float2*>(row + j * LD);
+          } else {
+            u[0] = row[j * LD];
+          }
+#pragma unroll
+          for (int h = 0; h < M / 4; ++h)
+            *reinterpret_cast<float4*>(v + 4 * h) = *reinterpret_cast<const float4*>(col + j * LD + 16 * h);
+#pragma unroll
+          for (int x = 0; x < R; ++x)
+#pragma unroll
+            for (int y = 0; y < M / 2; ++y)
+              acc[x][y] = __ffma2_rn(make_float2(u[x], u[x]), make_float2(v[2 * y], v[2 * y + 1]), acc[x][y]);
+        }
+      }
+      if (t + 1 < n_chunks) put(t + 1);
       __syncthreads();
     }
-    for (int e = tid; e < nj * (D / 4); e += 256) {
-      float4 x = reinterpret_cast<float4*>(work)[e];
-      const float4 m = *reinterpret_cast<const float4*>(mean_s + (e % (D / 4)) * 4);
-      x.x -= m.x; x.y -= m.y; x.z -= m.z; x.w -= m.w;
-      reinterpret_cast<float4*>(work)[e] = x;
-    }
-    __syncthreads();
-#pragma unroll 2
-    for (int jj = 0; jj < nj; ++jj) {
-      const float* x = work + jj * D;
-      float a[T], b[T];
+    // the quarters: 0 + 1 and 2 + 3 within a warp, the two sums through shared memory ([2][slot][E][E])
 #pragma unroll
-      for (int h = 0; h < T / 4; ++h) {
-        *reinterpret_cast<float4*>(a + 4 * h) = *reinterpret_cast<const float4*>(x + 64 * h + 4 * ty);
-        *reinterpret_cast<float4*>(b + 4 * h) = *reinterpret_cast<const float4*>(x + 64 * h + 4 * tx);
+    for (int x = 0; x < R; ++x)
+#pragma unroll
+      for (int y = 0; y < M / 2; ++y) {
+        acc[x][y].x += __shfl_xor_sync(0xffffffffu, acc[x][y].x, 16);
+        acc[x][y].y += __shfl_xor_sync(0xffffffffu, acc[x][y].y, 16);
       }
+    if (quarter % 2 == 0) {
+      float* to = work + ((quarter / 2 * kSlots + group / kParts) * E + rp) * E + c0;
 #pragma unroll
-      for (int r = 0; r < T; ++r)
+      for (int x = 0; x < R; ++x)
 #pragma unroll
-        for (int c = 0; c < T / 2; ++c)
-          acc[r][c] = __ffma2_rn(make_float2(a[r], a[r]), make_float2(b[2 * c], b[2 * c + 1]), acc[r][c]);
+        for (int h = 0; h < M / 4; ++h)
+          *reinterpret_cast<float4*>(to + (x / 4 * 16 + x % 4) * E + 16 * h) =
+              make_float4(acc[x][2 * h].x, acc[x][2 * h].y, acc[x][2 * h + 1].x, acc[x][2 * h + 1].y);
     }
     __syncthreads();
+    constexpr int kPieces = E * E / 4;
+    for (int e = tid; e < kSlots * kPieces; e += 256) {
+      const int bb = first + e / kPieces * n_cta + rank, at = e % kPieces;
+      if (bb >= kBlocks) break;                  // (and so are the slots behind it)
+      float4 x = add4(work4[e], work4[kSlots * kPieces + e]);
+      const float n = (float)Nk;
+      x.x /= n; x.y /= n; x.z /= n; x.w /= n;
+      const int xi = block_row(bb), xj = block_col(bb, xi), i = xi * E + at / (E / 4), j = xj * E + at % (E / 4) * 4;
+      *reinterpret_cast<float4*>(cov + i * D + j) = x;
+      if (xi != xj) {                            // the mirror image below the diagonal
+        cov[j * D + i] = x.x;
+        cov[(j + 1) * D + i] = x.y;
+        cov[(j + 2) * D + i] = x.z;
+        cov[(j + 3) * D + i] = x.w;
+      }
+    }
+    __syncthreads();
+    return first + kSlots * n_cta;
+  };
+  for (int first = 0; first < kBlocks;) {
+    const int per = ceil_div(kBlocks - first, n_cta);          // blocks that this CTA may still have
+    if (per > 2) first = pass(std::integral_constant<int, M>{}, first);
+    else if (per == 2) first = pass(std::integral_constant<int, M / 2>{}, first);
+    else first = pass(std::integral_constant<int, M / 4>{}, first);
   }
-  const float inv = 1.f / (float)Nk;
-#pragma unroll
-  for (int r = 0; r < T; ++r)
-#pragma unroll
-    for (int h = 0; h < T / 4; ++h) {
-      const float2 lo = acc[r][2 * h], hi = acc[r][2 * h + 1];
-      *reinterpret_cast<float4*>(cov + (size_t)((r / 4) * 64 + 4 * ty + r % 4) * D + 64 * h + 4 * tx) =
-          make_float4(lo.x * inv, lo.y * inv, hi.x * inv, hi.y * inv);
-    }
+  sync();
   if (n_cta > 1) {
-    cluster.sync();
-    // add the partial matrices, one strip per CTA, then gather the strips
-    constexpr int kPieces = D * D / 4;
-    const int per = ceil_div(kPieces, n_cta);
-    const int e0 = min(kPieces, rank * per), e1 = min(kPieces, e0 + per);
-    for (int e = e0 + tid; e < e1; e += 256) {
-      float4 y[8], r = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int x = 0; x < 8; ++x)
-        y[x] = x < n_cta ? reinterpret_cast<const float4*>(cluster.map_shared_rank(cov, x))[e] : r;
-#pragma unroll
-      for (int x = 0; x < 8; ++x) { r.x += y[x].x; r.y += y[x].y; r.z += y[x].z; r.w += y[x].w; }
-      reinterpret_cast<float4*>(work)[e - e0] = r;
-    }
-    cluster.sync();
+    // gather the other CTAs' blocks
 #pragma unroll 8
-    for (int e = tid; e < kPieces; e += 256)
-      reinterpret_cast<float4*>(cov)[e] = reinterpret_cast<const float4*>(cluster.map_shared_rank(work, e / per))[e % per];
-    cluster.sync();                              // the strips are read: `work` is free again, and a CTA may leave
-  } else {
-    __syncthreads();
+    for (int e = tid; e < D * P4; e += 256) {
+      const int x = e / P4 / E, y = piece * 4 / E, bi = min(x, y), bj = max(x, y);
+      const int owner = (4 * bi - bi * (bi - 1) / 2 + bj - bi) % n_cta;
+      if (owner != rank)
+        reinterpret_cast<float4*>(cov)[e] = reinterpret_cast<const float4*>(cluster.map_shared_rank(cov, owner))[e];
+    }
+    cluster.sync();                              // a CTA may leave once its blocks are read
   }
 
   // ---- Y = Qbar C_K and the row sums of Y o Qbar; thread (ty, tx) owns query blocks ty + 16 a and columns
@@ -365,7 +426,8 @@ __global__ void __launch_bounds__(256, 2) thresholds_moments_kernel(WsPtrs ws, i
   auto rows = [&](auto a_c, int i0) {
     constexpr int A = decltype(a_c)::value;
     const int nq = min(min(16 * A, kMomentRows), i_end - i0);
-    stage(ws.qbar + ((size_t)bh * Nq + i0) * D, nq);
+#pragma unroll 4
+    for (int e = tid; e < nq * P4; e += 256) work4[e] = reinterpret_cast<const float4*>(ws.qbar + ((size_t)bh * Nq + i0) * D)[e];
     __syncthreads();
     const float* q_row[A];                       // (rows past the last repeat it and are not stored)
 #pragma unroll
@@ -502,6 +564,25 @@ __global__ void __launch_bounds__(256) tau_diag_kernel(WsPtrs ws, int Nq, float 
   }
 }
 
+// CTAs per head of thresholds_moments_kernel: the size with the least time.  `cycles` is a CTA's time in thousands (591 x 591
+// blocks, d = 128; other sizes are in much the same proportions).  As many CTAs as find an SM of their own run at that pace:
+// clusters of 1 and 2 fill the GPU, clusters of 3 to 6 about 17/20 of it, and of clusters of 8 no more than 14 are placed at
+// once.  Two CTAs on an SM share its FMA pipes and take 1.8 times as long.  us with the size taken / others: 40 heads x 591 blocks
+// (3) 58 / 6: 64, 2: 84; 16 x 591 (6) 41 / 8: 52; 48 x 300 (5) 35 / 2: 46; 80 x 300 (3) 57 / 1: 78.
+static int cluster_size(int heads, int sms) {
+  struct { int n, cycles; } const sizes[] = {{8, 46}, {6, 53}, {5, 58}, {4, 82}, {3, 95}, {2, 141}, {1, 268}};
+  int best = 1;
+  long long least = -1;
+  for (const auto& s : sizes) {
+    const long long ctas = (long long)heads * s.n;
+    const long long fit = s.n == 8 ? 8 * (14 * sms / 148) : (s.n > 2 ? sms * 17 / 20 : sms);
+    if (s.n > 1 && ctas > 2 * fit) continue;     // (would wait for its turn)
+    const long long time = ctas <= fit ? 10LL * s.cycles : 18LL * s.cycles;
+    if (least < 0 || time < least) { least = time; best = s.n; }
+  }
+  return best;
+}
+
 template <int D>
 static cudaError_t thresholds_impl(const Problem& p, const WsPtrs& ws, cudaStream_t stream, int* n_launches) {
   const bool diag = p.estimator == SOL_EST_DIAGONAL;
@@ -517,15 +598,11 @@ static cudaError_t thresholds_impl(const Problem& p, const WsPtrs& ws, cudaStrea
     if (n_launches) *n_launches += 2;
     return cudaGetLastError();
   }
-  // One cluster per head, as large as leaves every CTA an SM of its own with room for the clusters to be packed
-  // into GPCs: two CTAs on an SM share its FMA pipes and take twice as long.  40 heads x 591 blocks: clusters of 2 / 3 /
-  // 4 / 7 take 80 / 60 / 82 / 77 us; 24 heads x 300: 4 / 5 / 6 take 27 / 24 / 38 us.
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const int fit = sms * 17 / 20 / p.BH;
-  const int n_cta = fit < 1 ? 1 : (fit > 8 ? 8 : fit);
+  const int n_cta = cluster_size(p.BH, sms);
   if (n_launches) *n_launches += 1;
   return launch_after(thresholds_moments_kernel<D>, dim3(n_cta, p.BH), 256, moments_smem<D>(), moments_smem<D>(), n_cta, stream, ws, p.Nq, p.Nk,
                       p.scale, p.beta);

@@ -22,10 +22,13 @@ def _pooled(BH, N, d, block, seed):
     return q, k, v
 
 
-# Nk: one block, sizes at which the one-pass kernel's shared memory is just below and above 48 KB, the sizes next to its 128, row steps of 32 / 64 / 88 per CTA of a cluster, and
-# clusters of 8, 7 (40 heads), 1 (400 heads)
+# Nk: one block, sizes at which the one-pass kernel's shared memory is just below and above 48 KB, the sizes next to its 128, row
+# steps of 32 / 64 / 88 per CTA of a cluster, ragged chunks of keys, and clusters of 8 (up to 14 heads), 6 (20), 5 (25, 48), 4 (30),
+# 3 (40, 80), 2 (60, 100) and 1 (400 heads)
 @pytest.mark.parametrize("BH,n_blocks,d", [(1, 1, 64), (3, 17, 128), (2, 66, 128), (2, 73, 128), (2, 90, 128), (2, 92, 128), (2, 128, 64), (2, 128, 128), (2, 129, 64), (2, 129, 128),
-                                           (3, 300, 128), (40, 260, 128), (40, 591, 64), (400, 130, 64), (1, 1500, 128)])
+                                           (3, 300, 128), (40, 260, 128), (40, 591, 64), (400, 130, 64), (1, 1500, 128),
+                                           (14, 161, 64), (20, 193, 128), (25, 160, 128), (30, 131, 64), (48, 140, 128), (60, 150, 64),
+                                           (80, 133, 128), (100, 191, 64), (400, 129, 128)])
 @pytest.mark.parametrize("estimator", ["moments", "diagonal"])
 def test_thresholds(sb, BH, n_blocks, d, estimator):
     block = 64 if n_blocks < 1000 else 16
