@@ -193,9 +193,20 @@ typedef struct {
   int32_t layout;                               /* SOL_LAYOUT_* of q, k, v and out (0 = [B,H,N,d]) */
   int32_t routing;                              /* SOL_ROUTING_* (0 = inside the fused kernel)   */
 } sol_attn_args;
-/* Everything sol_attn_forward_ex enqueues is ordinary work on `stream` (a memset of the status words
- * and kernels), so the call may be captured into a CUDA graph and replayed; sol_attn_forward_host may
- * not (it creates events and uses streams of its own). */
+/* Everything sol_attn_forward_ex enqueues is work on `stream` (kernels, and a memset of the status words in
+ * SOL_MODE_DENSE or with skip_pool), so the call may be captured into a CUDA graph and replayed;
+ * sol_attn_forward_host may not (it creates events and uses streams of its own).
+ *
+ * The kernels of a call, and those of sol_attn_thresholds and sol_attn_route_mask, are launched with programmatic
+ * stream serialization: each may be put in place while the one before it still runs, and waits for it on the
+ * device.  Work that follows on the stream in the ordinary way sees everything finished.  A kernel of the caller's
+ * that is itself launched with that attribute right behind sol_attn_pool or sol_attn_thresholds has to execute
+ * the grid dependency wait (griddepcontrol.wait) before it reads mu, sigma or tau.
+ *
+ * Heads are independent.  The pooled tensors, mu, sigma and tau of a head are the same, bit for bit, in whatever
+ * group of heads it is called.  So are its routing and output with 128-token blocks; with 64-token blocks, and in
+ * SOL_MODE_DENSE, calls of different sizes go to different kernels, which agree up to rounding (a proxy score within
+ * fp32 rounding of its threshold, the last bf16 bit of the output). */
 sol_status_t sol_attn_forward_ex(const sol_attn_args* args /* host */);
 
 /* End-to-end convenience for callers whose tensors live in HOST memory ([B,H,N,d] layout;

@@ -462,7 +462,9 @@ struct Cursor {
 
 // One issuing warp per stream s.  S = Q K^T of a tile goes to one of the stream's two score buffers, P V of
 // the tile that was there before having been issued first, so that the new scores may overwrite P without a
-// completion signal in between.
+// completion signal in between.  That is an assumption: MMAs that one thread issues run in the order of issue, also
+// where shape and accumulator differ (the order that is promised is that of MMAs of one shape on one accumulator).  Other
+// attention kernels for this architecture make it too, and every output test of this one would show where it failed.
 //
 // The warp runs in lockstep and one elected lane issues: with warp-uniform control flow and operands the
 // compiler keeps descriptors and addresses in uniform registers, where the MMA instruction wants them.
@@ -664,7 +666,7 @@ __device__ void softmax_role(Shared<C>& sm, const Params& p, uint32_t tmem, int 
   const int row = warp_in_group * 32 + lane;                 // row of the query tile
   const int u = s * kSub + row / kBlk;                       // query block of the item (the same for a whole warp)
   const float sl2 = p.scale * 1.4426950408889634f;
-  uint32_t g = 0, n_rec = 0, n_item = 0;                     // tiles, records and work items so far
+  uint32_t g = 0, n_rec = 0;                                 // tiles and records so far
   uint32_t g_item0 = 0;                                      // first tile of the work item
   float m_used = -INFINITY, l = 0.f;
   bool started = false;
@@ -846,7 +848,6 @@ __device__ void softmax_role(Shared<C>& sm, const Params& p, uint32_t tmem, int 
           }
         }
       }
-      ++n_item;
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&sm.rec_empty[r]);

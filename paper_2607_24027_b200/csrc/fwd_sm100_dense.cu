@@ -187,6 +187,8 @@ __device__ void mma_role(Shared& sm, const Params& p, unsigned char* sQ, unsigne
           // (test hook: a withheld completion signal makes the bounded waits on it run out)
           if (s == 1 && (int)g != p.withhold_tile) mma_commit(&sm.kv_empty[v_slot]);
         }
+        // (the scores overwrite P behind a P V that has been issued, not completed: MMAs of one thread are assumed to run in
+        //  the order of issue, also where shape and accumulator differ)
         if (next) scores(s, k_slot);
         if (leader) {
           // Q is free behind the last scores that read it (of this item, or of a next item with one tile)

@@ -122,17 +122,22 @@ row_select_warp_kernel(const float* __restrict__ map, long long n_rows, int Nk, 
       const double x = __shfl_up_sync(0xffffffffu, run, o);
       if (lane >= o) run += x;
     }
-    const double total = __shfl_sync(0xffffffffu, run, 31);
+    // (the total of the last lane with any mass: the lanes behind it add nothing, but in another order)
+    const unsigned live = __ballot_sync(0xffffffffu, local != 0.0);
+    const double total = __shfl_sync(0xffffffffu, run, live ? 31 - __clz(live) : 0);
     double before_lane = __shfl_up_sync(0xffffffffu, run, 1);
     if (lane == 0) before_lane = 0.0;
     const double need = (double)param * total;
-    // the first c with mass(c) >= need; mass(c) = sum of the first c blocks
+    // the first c with mass(c) >= need; mass(c) = sum of the first c blocks.  The scan says in which lane that is; the
+    // lane's own running sum may end a rounding below the scan's, and then its last block with any mass is the one.
     int first = Nk;
-    if (before_lane < need) {
+    if (before_lane < need && need <= run) {
       double mass = before_lane;
       for (int j = j0; j < min(j0 + kPer, Nk); ++j) {
-        mass += exp((double)val[warp][j] - (double)top);
-        if (mass >= need) { first = j + 1; break; }
+        const double x = exp((double)val[warp][j] - (double)top);
+        mass += x;
+        if (x != 0.0) first = j + 1;
+        if (mass >= need) break;
       }
     }
     c = __reduce_min_sync(0xffffffffu, first);
@@ -212,11 +217,14 @@ __global__ void __launch_bounds__(256) row_select_kernel(const float* __restrict
     const double need = (double)param * total_s;
     double run = part[threadIdx.x];
     int first = Nk;
-    // the first c with mass(c) >= need; mass(c) = sum of the first c blocks
-    if (run < need) {
+    // the first c with mass(c) >= need; mass(c) = sum of the first c blocks.  The scan says whose block that is; the
+    // thread's own running sum may end a rounding below the scan's, and then its last block with any mass is the one.
+    if (run < need && need <= run + local) {
       for (int j = j0; j < j1; ++j) {
-        run += exp((double)val[j] - (double)top);
-        if (run >= need) { first = j + 1; break; }
+        const double x = exp((double)val[j] - (double)top);
+        run += x;
+        if (x != 0.0) first = j + 1;
+        if (run >= need) break;
       }
     }
     if (first < Nk) atomicMin(&cut, first);

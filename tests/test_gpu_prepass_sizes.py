@@ -81,6 +81,25 @@ def test_materialised_order(sb, BH, nq, nk, d, aligned):
         assert np.array_equal(tau[0].cpu().numpy().astype(np.float64), t)
 
 
+@pytest.mark.parametrize("nk", [33, 250, 256, 700, 1024, 1500, 5000])
+def test_top_p_of_one_ends_with_the_mass(sb, nk):
+    """p = 1 keeps the blocks that have any share: the running sum of a lane may round differently from the scan over the
+    lanes, which must not make the row miss its end and keep everything."""
+    rows, d = 400, 32
+    rng = np.random.default_rng(nk)
+    some = rng.integers(1, nk, rows)                               # blocks with mass; the others' exponentials are zero
+    scores = np.where(np.arange(nk) < some[:, None], rng.uniform(-3, 3, (rows, nk)), -1e4).astype(np.float32)
+    for row in scores:
+        rng.shuffle(row)
+    qb, kc = torch.zeros(1, rows, 1, d), torch.zeros(1, rows, nk, d)
+    qb[..., 0] = 1.0
+    kc[0, :, :, 0] = torch.from_numpy(scores)                     # one row of scores per head
+    pm, counts, tau = torch.empty(1, rows, 1, nk), torch.empty(1, rows, 1, dtype=torch.int32), torch.empty(1, rows, 1)
+    qb, kc, pm, counts, tau = (x.cuda() for x in (qb, kc, pm, counts, tau))
+    sb.sol_attn_route_materialized(qb, kc, sb.SOL_ROUTE_TOPP, 1.0, pm, tau, counts=counts, scale=1.0)
+    assert np.array_equal(counts.cpu().numpy()[0, :, 0], some)
+
+
 @pytest.mark.parametrize("n_q,n_k", [(1, 1), (127, 63), (128, 64), (129, 65), (257, 97), (64, 591)])
 def test_mask_bits(sb, n_q, n_k):
     """Bits of ragged tiles, against the same comparison in 64 bits; block_q and block_k differ so that Nq and Nk do."""
