@@ -20,7 +20,7 @@
 //
 // 40 heads x 32 760 tokens, d = 128: 19.9 ms against 20.0 ms with one query tile per CTA (19.7 with the row sum of the
 // unrounded weights, see softmax_role; the part is at its 1 kW limit in all three); d = 64, 40 x 16 000: 3.69 ms against
-// 3.93 ms.  A pair of tiles takes 3 400 cycles, of which the tensor core needs 2 048: a tile's softmax, P V and next Q K^T
+// 3.93 ms.  A pair of tiles takes 3 460 cycles, of which the tensor core needs 2 048: a tile's softmax, P V and next Q K^T
 // follow one another, and beside the other tile's the three take that long.
 // Every wait is bounded, as in the other kernels.
 #include <atomic>
