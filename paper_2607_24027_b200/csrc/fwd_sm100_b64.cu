@@ -861,8 +861,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 fwd_sm100_b64_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_kc,
                  const __grid_constant__ CUtensorMap tm_vm, const Params p) {
-  extern __shared__ unsigned char smem_raw[];
-  unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  extern __shared__ __align__(1024) unsigned char smem_raw[];   // (see fwd_sm100.cu)
+  unsigned char* base = smem_raw;
   unsigned char* sQ = base;
   unsigned char* sKV = base + 2 * C::kQBytes;
   Shared<C>& sm = *reinterpret_cast<Shared<C>*>(base + 2 * C::kQBytes + 2 * kStages * C::kTileBytes);
@@ -914,7 +914,7 @@ fwd_sm100_b64_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
 
 template <class C>
 cudaError_t launch_instance(const Problem& p, const Maps& m, const Params& prm, int grid, cudaStream_t stream) {
-  const size_t smem = 1024 + 2 * C::kQBytes + 2 * kStages * C::kTileBytes + sizeof(Shared<C>);
+  const size_t smem = 2 * C::kQBytes + 2 * kStages * C::kTileBytes + sizeof(Shared<C>);
   auto kernel = p.routing == SOL_ROUTING_PREPASS && p.mode != SOL_MODE_DENSE ? fwd_sm100_b64_kernel<C, true>
                                                                             : fwd_sm100_b64_kernel<C, false>;
   return launch_after(kernel, dim3(grid), kThreads, smem, smem, 0, stream, m.q, m.k, m.v, m.kc, m.vm, prm);

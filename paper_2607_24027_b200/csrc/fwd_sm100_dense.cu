@@ -55,7 +55,7 @@ struct Shared {
   int abort_flag;
 };
 
-#define WAIT(bar, parity) mbar_wait((bar), (parity), &sm.abort_flag, p.wait_limit)
+#define WAIT(bar, parity) mbar_wait_inline((bar), (parity), &sm.abort_flag, p.wait_limit)
 #define WAIT_ALL(bar, parity) __all_sync(0xffffffffu, WAIT(bar, parity))
 
 // Work items are dealt out round robin: they all cost the same.
@@ -109,10 +109,10 @@ __device__ void producer_role(Shared& sm, const Params& p, unsigned char* sQ, un
     // let copies that are still in flight land before the CTA's shared memory goes away (not cut short by the flag)
     int never = 0;
     for (int s = 0; s < 2; ++s)
-      if (n_q[s] > 0) mbar_wait(&sm.q_full[s], (n_q[s] - 1) & 1, &never, p.wait_limit);
+      if (n_q[s] > 0) mbar_wait_inline(&sm.q_full[s], (n_q[s] - 1) & 1, &never, p.wait_limit);
     for (uint32_t back = 0; back < kSlots && back < m; ++back) {
       const uint32_t n = m - 1 - back;
-      mbar_wait(&sm.kv_full[n % kSlots], (n / kSlots) & 1, &never, p.wait_limit);
+      mbar_wait_inline(&sm.kv_full[n % kSlots], (n / kSlots) & 1, &never, p.wait_limit);
     }
   }
 }
@@ -205,7 +205,7 @@ __device__ void mma_role(Shared& sm, const Params& p, unsigned char* sQ, unsigne
     // TMEM must not be released while MMAs are still writing to it: wait (bounded) behind everything issued
     if (leader) mma_commit(&sm.mma_drain);
     int never = 0;
-    mbar_wait(&sm.mma_drain, 0, &never, p.wait_limit);
+    mbar_wait_inline(&sm.mma_drain, 0, &never, p.wait_limit);
   }
 }
 
@@ -376,8 +376,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 fwd_sm100_dense_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                        const __grid_constant__ CUtensorMap tm_v, const Params p, int block) {
   using C = Cfg<D>;
-  extern __shared__ unsigned char smem_raw[];
-  unsigned char* sQ = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  extern __shared__ __align__(1024) unsigned char smem_raw[];   // (see fwd_sm100.cu)
+  unsigned char* sQ = smem_raw;
   unsigned char* sKV = sQ + 2 * C::kTileBytes;
   Shared& sm = *reinterpret_cast<Shared*>(sKV + kSlots * C::kTileBytes);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -427,7 +427,7 @@ cudaError_t launch_instance(const Problem& p, const Maps& m, const Params& prm, 
     if (a.numRegs < kRegsLaunch) return cudaErrorInvalidConfiguration;
     enough = true;
   }
-  const size_t smem = 1024 + (2 + kSlots) * Cfg<D>::kTileBytes + sizeof(Shared);
+  const size_t smem = (2 + kSlots) * Cfg<D>::kTileBytes + sizeof(Shared);
   return launch_after(fwd_sm100_dense_kernel<D>, dim3(grid), kThreads, smem, smem, 0, stream, m.q, m.k, m.v, prm, p.block_q);
 }
 

@@ -61,9 +61,31 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
 // Bounded wait on an mbarrier phase.  Gives up after ~`limit` SM clocks (kWaitCycles unless the
 // caller says otherwise) or as soon as another thread of the CTA has flagged an abort; returns
 // false in that case.
+//
+// Only the first look is inline.  The fused kernels have four to six roles with code of their own in 45 to 65 KB, more than an SM's
+// instruction caches hold beside the unrolled softmax loop, and a role that runs a few hundred instructions once per
+// tile finds them evicted: the less of it, the sooner a role is through (us, spinning inline / out of line: 24 heads x 4096 tokens
+// 105.5 / 103.5, with 77 text tokens as a batch of two 242 / 239, 64-token blocks 16 x 11 160 d = 64 318 / 312).
 constexpr long long kWaitCycles = 4000000000LL;   // about 2-3 s of SM clocks
+static __device__ __noinline__ bool mbar_keep_waiting(uint64_t* bar, uint32_t parity, volatile int* abort_flag, long long limit) {
+  const long long t0 = clock64();
+  uint32_t spins = 0;
+  while (!mbar_try_wait(bar, parity)) {
+    if ((++spins & 0x3ffu) == 0) {
+      if (*abort_flag) return false;
+      if (clock64() - t0 > limit) return false;
+    }
+  }
+  return true;
+}
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                           long long limit = kWaitCycles) {
+  return mbar_try_wait(bar, parity) || mbar_keep_waiting(bar, parity, abort_flag, limit);
+}
+
+// The same without the call, for the dense kernel, whose split of the registers leaves no room for one.
+__device__ __forceinline__ bool mbar_wait_inline(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                          long long limit) {
   if (mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();
   uint32_t spins = 0;
