@@ -2,7 +2,7 @@
 //
 // The tensor core's query tile has 128 rows at full rate (an M = 64 MMA takes as long), so one query block
 // of 64 tokens per tile would leave half of the matrix and softmax work unused.  Here a persistent CTA of
-// 384 threads works on up to 256 consecutive query rows of one head at a time, as two STREAMS of 128 rows,
+// 448 threads works on up to 256 consecutive query rows of one head at a time, as two STREAMS of 128 rows,
 // i.e. four query blocks.  Each stream has its own query tile, score buffers, accumulator, softmax warpgroup
 // and MMA-issuing warp; the two share every K and V tile that both of them need.  The query blocks route
 // independently: a tile is computed for a stream when either of its two blocks wants it, the warps of a
@@ -27,8 +27,8 @@
 //   producer (warp 9, one lane) reads the records and issues TMA loads: one approximate tile per
 //                      chunk (KC chunk, mean-V chunk) and K_j / V_j ONLY for key blocks that some
 //                      query block of the item routed.
-//   mma      (warps 10, 11) one issuing warp per stream, with two score buffers: the scores of a tile are
-//                      computed while the one before is in its softmax.
+//   mma      (warps 10-13) two issuing warps per stream, one for the scores and one for P V, with two score
+//                      buffers: the scores of a tile are computed while the one before is in its softmax.
 //   softmax  (warps 0-3 and 4-7) warpgroup s serves stream s; thread = query row, with its running
 //                      (m, l).  Both branches of the method update the same state: an approximate tile
 //                      is an ordinary tile whose columns carry the bias log2(n_j) (Eqs. 9-10:
@@ -61,7 +61,8 @@ constexpr uint32_t kSubMask = (1u << kSub) - 1;
 constexpr int kStages = 4;
 constexpr int kGroup = 16;                       // pooled keys per router staging buffer
 constexpr int kRecords = 4;                      // ring of routing records
-constexpr int kWarpMma = 10;                     // one MMA-issuing warp per stream
+constexpr int kWarpQK = 10, kWarpPV = 12;        // one warp each per stream
+constexpr int kThreads64 = 448;
 constexpr int kTmemS = 0, kTmemO = 256;
 
 // Compile-time shape of one kernel instance.
@@ -110,7 +111,7 @@ struct Shared {
   uint64_t p_full[2][2];        // its P is in TMEM
   uint64_t pv_done[2][2];       // its P V is in the accumulator
   uint64_t kc_full[2];          // router staging buffers filled
-  uint64_t mma_drain[2];        // abort path only: all MMAs issued by a role have retired
+  uint64_t mma_drain[4];        // abort path only: all MMAs issued by a role have retired
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -452,169 +453,137 @@ __device__ void producer_role(Shared<C>& sm, const Params& p, unsigned char* sQ,
 }
 
 // ------------------------------------------------------------------------------------------------
-// A stream's position in the records, once for the K side (score GEMMs) and once for the V side.
-struct Cursor {
-  uint32_t n_rec = 0, n_item = 0;              // records and work items so far
-  uint32_t slot = 0, par = 0;                  // ring position of the tile
-  const Record* rec = nullptr;                 // the open record
-  int e = 0, n = 0, last = -1;                 // its descriptors; the stream's last one
-  uint32_t use = 0;                            // query blocks of the stream that use the tile
-  bool exists = false, last_chunk = false;
-  bool fresh = false;                          // start of a work item not dealt with yet
-};
-
-// One issuing warp per stream s.  S = Q K^T of a tile goes to one of the stream's two score buffers, P V of
-// the tile that was there before having been issued first, so that the new scores may overwrite P without a
-// completion signal in between.  That is an assumption: MMAs that one thread issues run in the order of issue, also
-// where shape and accumulator differ (the order that is promised is that of MMAs of one shape on one accumulator).  Other
-// attention kernels for this architecture make it too, and every output test of this one would show where it failed.
+// Two issuing warps per stream s, one for the score GEMMs and one for the value GEMMs.  A warp that did both had to look at
+// every barrier in turn without ever sleeping (each side may have something to release that the other waits for): 304 us at
+// 16 heads x 11 160 tokens, d = 64, keep-or-drop, where two that simply wait take 271, although a score GEMM now needs
+// a completion signal of the P V whose buffer it takes over.
 //
-// The warp runs in lockstep and one elected lane issues: with warp-uniform control flow and operands the
+// The warps run in lockstep and one elected lane issues: with warp-uniform control flow and operands the
 // compiler keeps descriptors and addresses in uniform registers, where the MMA instruction wants them.
 // Every wait is made uniform by a vote; a lane that fell behind could otherwise miss a phase.
 //
 // A tile that only the other stream uses is released as soon as it has landed (not earlier: an arrival
-// before that could be taken for one of the slot's previous tile).  K and V are passed on by cursors of
-// their own, and the warp never sleeps on one side while the other may have something to release.
+// before that could be taken for one of the slot's previous tile).
+#define NEED(bar, parity) if (!__all_sync(0xffffffffu, WAIT(bar, parity))) { ok = false; break; }
+
+// Abort path: TMEM must not be released while MMAs are still writing to it, so the role asks for a
+// completion signal behind everything it has issued and waits for it (bounded).
 template <class C>
-__device__ void mma_role(Shared<C>& sm, const Params& p, unsigned char* sQ, unsigned char* sKV, uint32_t tmem, int s) {
+__device__ void drain_mmas(Shared<C>& sm, const Params& p, bool ok, bool leader, int which) {
+  if (!ok && leader) flag_abort(sm, p, 300 + which);
+  __syncwarp();
+  if (sm.abort_flag) {
+    if (leader) mma_commit(&sm.mma_drain[which]);
+    int never = 0;
+    mbar_wait(&sm.mma_drain[which], 0, &never, p.wait_limit);
+  }
+}
+
+// S = Q K^T of the stream's tiles, alternating between its two score buffers
+template <class C>
+__device__ void mma_qk_role(Shared<C>& sm, const Params& p, unsigned char* sQ, unsigned char* sKV, uint32_t tmem, int s) {
   constexpr int kD = C::kD, kTileBytes = C::kTileBytes;
-  const unsigned full = 0xffffffffu;
   const long long wait_limit = p.wait_limit;
   const uint32_t idesc_qk = make_idesc_bf16(kRowsQ, kBlk, false, false);
-  const uint32_t idesc_pv = make_idesc_bf16(kRowsQ, kD, false, true);
   const uint32_t q_lo = (smem_addr(sQ + s * C::kQBytes) >> 4) | (1u << 16);
   const uint32_t k_lo0 = (smem_addr(sKV) >> 4) | (1u << 16);
+  const uint32_t t_s0 = tmem + kTmemS + s * 2 * kBlk;
+  const bool leader = elect_one();
+  uint32_t slot = 0, par = 0, n_item = 0, n = 0;   // ring position; work items with the stream; tiles issued
+  bool fresh = false, ok = true;               // the work item's Q has not been waited for
+  for (uint32_t n_rec = 0; ok; ++n_rec) {
+    const uint32_t r = n_rec % kRecords;
+    NEED(&sm.rec_full[r], (n_rec / kRecords) & 1)
+    const Record& rec = sm.rec[r];
+    if (rec.work < 0) break;
+    const int n_desc = rec.n, last = rec.last[s];
+    const bool exists = (rec.valid >> (s * kSub)) & 1, last_chunk = (rec.flags & kRecLast) != 0;
+    if (exists && (rec.flags & kRecFirst)) { fresh = true; ++n_item; }
+    for (int e = 0; e < n_desc; ++e) {
+      const uint32_t use = (rec.desc[e] >> (s * kSub)) & kSubMask;
+      NEED(&sm.k_full[slot], par)
+      if (use) {
+        if (fresh) { NEED(&sm.q_full[s], (n_item - 1) & 1) }
+        fresh = false;
+        const uint32_t x = n & 1;
+        // P overwrites S: the P V of the buffer's tile before must have read P
+        if (n >= 2) { NEED(&sm.pv_done[s][x], ((n - 2) >> 1) & 1) }
+        tc_fence_after();
+        const uint32_t k_lo = k_lo0 + slot * (kTileBytes >> 4);
+#pragma unroll
+        for (int ks = 0; ks < kD / 16; ++ks) {
+          // K-step ks: 16 channels = 32 bytes inside box ks / 4
+          const uint32_t off_q = ((ks / 4) * C::kQBoxBytes + (ks % 4) * 32) >> 4;
+          const uint32_t off_k = ((ks / 4) * C::kBoxBytes + (ks % 4) * 32) >> 4;
+          const uint64_t da = desc_from_lo(q_lo + off_q), db = desc_from_lo(k_lo + off_k);
+          if (leader) mma_ss(t_s0 + x * kBlk, da, db, idesc_qk, ks > 0);
+        }
+        if (leader) {
+          mma_commit(&sm.s_full[s][x]);
+          mma_commit(&sm.k_empty[slot]);
+          if (last_chunk && e == last) mma_commit(&sm.q_empty[s]);
+        }
+        ++n;
+      } else if (leader) {
+        mbar_arrive(&sm.k_empty[slot]);
+      }
+      if (++slot == kStages) { slot = 0; par ^= 1; }
+    }
+    if (!ok) break;
+    if (exists && last_chunk && last < 0) {    // an item without a tile in its last chunk hands Q back here
+      if (fresh) {                             // nothing has read Q
+        NEED(&sm.q_full[s], (n_item - 1) & 1)
+        if (leader) mbar_arrive(&sm.q_empty[s]);
+        fresh = false;
+      } else if (leader) {
+        mma_commit(&sm.q_empty[s]);
+      }
+    }
+    __syncwarp();
+    if (leader) mbar_arrive(&sm.rec_empty[r]);
+  }
+  drain_mmas(sm, p, ok, leader, s);
+}
+
+// O (+)= P V of the stream's tiles
+template <class C>
+__device__ void mma_pv_role(Shared<C>& sm, const Params& p, unsigned char* sKV, uint32_t tmem, int s) {
+  constexpr int kD = C::kD, kTileBytes = C::kTileBytes;
+  const long long wait_limit = p.wait_limit;
+  const uint32_t idesc_pv = make_idesc_bf16(kRowsQ, kD, false, true);
   // V is the MN-major operand: its 64-channel boxes are C::kBoxBytes apart (leading offset), groups of
   // 8 key rows 1024 bytes apart; a K-step of 16 keys advances the start by 2048 bytes.
   const uint32_t v_lo0 = (smem_addr(sKV + kStages * kTileBytes) >> 4) | ((uint32_t)(C::kBoxBytes >> 4) << 16);
   const uint32_t t_s0 = tmem + kTmemS + s * 2 * kBlk, t_o = tmem + kTmemO + s * kD;
   const bool leader = elect_one();
-  Cursor ck, cv;
-  uint32_t n_qk = 0, n_pv = 0;                 // tiles whose Q K^T / P V has been issued
+  uint32_t slot = 0, par = 0, n = 0;
   uint32_t n_acc = 0;                          // work items with a tile of the stream
   uint32_t started = 0;                        // query blocks of the stream whose accumulator holds something
-  auto ready = [&](uint64_t* bar, uint32_t parity) { return __all_sync(full, mbar_test_wait(bar, parity)) != 0; };
-  auto open = [&](Cursor& c) {                 // the next record, which is there
-    const Record& rec = sm.rec[c.n_rec % kRecords];
-    c.rec = &rec;
-    c.e = 0;
-    c.n = rec.n;
-    c.last = rec.last[s];
-    c.last_chunk = (rec.flags & kRecLast) != 0;
-    c.exists = (rec.valid >> (s * kSub)) & 1;
-    if (c.exists && (rec.flags & kRecFirst)) {
-      c.fresh = true;
-      ++c.n_item;
-    }
-    if (c.n > 0) c.use = (rec.desc[0] >> (s * kSub)) & kSubMask;
-  };
-  auto next_tile = [&](Cursor& c) {
-    if (++c.slot == kStages) { c.slot = 0; c.par ^= 1; }
-    if (++c.e < c.n) c.use = (c.rec->desc[c.e] >> (s * kSub)) & kSubMask;
-  };
-  auto close = [&](Cursor& c) {
-    if (leader) mbar_arrive(&sm.rec_empty[c.n_rec % kRecords]);
-    c.rec = nullptr;
-    ++c.n_rec;
-  };
-  bool ok = true;
-  bool k_here = false, k_end = false;          // the K tile at the cursor can be used; no more tiles
-  uint32_t idle = 0;
-  long long t0 = 0;
-  for (;;) {
-    bool moved = false;
-    // ---- K side.  The next tile's K is looked for ahead of time, so that the score GEMM follows the P V
-    //      whose buffer it takes over without another look at a barrier; passing on what the stream does not use.
-    if (!k_here && !k_end) {
-      if (!ck.rec) {
-        if (ready(&sm.rec_full[ck.n_rec % kRecords], (ck.n_rec / kRecords) & 1)) {
-          if (sm.rec[ck.n_rec % kRecords].work < 0) k_end = true;
-          else open(ck);
-          moved = true;
+  bool fresh = false, ok = true;
+  for (uint32_t n_rec = 0; ok; ++n_rec) {
+    const uint32_t r = n_rec % kRecords;
+    NEED(&sm.rec_full[r], (n_rec / kRecords) & 1)
+    const Record& rec = sm.rec[r];
+    if (rec.work < 0) break;
+    const int n_desc = rec.n;
+    if (((rec.valid >> (s * kSub)) & 1) && (rec.flags & kRecFirst)) fresh = true;
+    for (int e = 0; e < n_desc; ++e) {
+      const uint32_t use = (rec.desc[e] >> (s * kSub)) & kSubMask;
+      NEED(&sm.v_full[slot], par)
+      if (use) {
+        if (fresh) {
+          // the first P V of a work item overwrites O: the epilogue of the last item with a tile must have read it
+          if (n_acc > 0) { NEED(&sm.o_free[s], (n_acc - 1) & 1) }
+          started = 0;
+          ++n_acc;
         }
-      } else if (ck.e == ck.n) {
-        // (an item without a tile in its last chunk hands Q back here)
-        bool done = true;
-        if (ck.exists && ck.last_chunk && ck.last < 0) {
-          if (ck.fresh) done = ready(&sm.q_full[s], (ck.n_item - 1) & 1);
-          if (done && leader) {
-            if (ck.fresh) mbar_arrive(&sm.q_empty[s]);       // nothing has read Q
-            else mma_commit(&sm.q_empty[s]);
-          }
-          if (done) ck.fresh = false;
-        }
-        if (done) { close(ck); moved = true; }
-      } else if (ready(&sm.k_full[ck.slot], ck.par)) {
-        if (!ck.use) {
-          if (leader) mbar_arrive(&sm.k_empty[ck.slot]);
-          next_tile(ck);
-          moved = true;
-        } else if (!ck.fresh || ready(&sm.q_full[s], (ck.n_item - 1) & 1)) {
-          ck.fresh = false;
-          k_here = true;
-          moved = true;
-        }
-      }
-    }
-    if (k_here && n_qk - n_pv < 2) {
-      tc_fence_after();
-      const uint32_t k_lo = k_lo0 + ck.slot * (kTileBytes >> 4);
-      const uint32_t d_s = t_s0 + (n_qk & 1) * kBlk;
-#pragma unroll
-      for (int ks = 0; ks < kD / 16; ++ks) {
-        // K-step ks: 16 channels = 32 bytes inside box ks / 4
-        const uint32_t off_q = ((ks / 4) * C::kQBoxBytes + (ks % 4) * 32) >> 4;
-        const uint32_t off_k = ((ks / 4) * C::kBoxBytes + (ks % 4) * 32) >> 4;
-        const uint64_t da = desc_from_lo(q_lo + off_q), db = desc_from_lo(k_lo + off_k);
-        if (leader) mma_ss(d_s, da, db, idesc_qk, ks > 0);
-      }
-      if (leader) {
-        mma_commit(&sm.s_full[s][n_qk & 1]);
-        mma_commit(&sm.k_empty[ck.slot]);
-        if (ck.last_chunk && ck.e == ck.last) mma_commit(&sm.q_empty[s]);
-      }
-      ++n_qk;
-      k_here = false;
-      next_tile(ck);
-      moved = true;
-    }
-    // ---- V side
-    if (!cv.rec) {
-      // (a record that the K side has opened is there for the V side too; in one without a tile of this
-      //  stream the V side may be done first, and must not run on into a record that is not written yet)
-      if ((int)(ck.n_rec - cv.n_rec) > 0 || (cv.n_rec == ck.n_rec && ck.rec)) { open(cv); moved = true; }
-    } else if (cv.e == cv.n) {
-      close(cv);
-      moved = true;
-    } else if (!cv.use) {
-      if (ready(&sm.v_full[cv.slot], cv.par)) {
-        if (leader) mbar_arrive(&sm.v_empty[cv.slot]);
-        next_tile(cv);
-        moved = true;
-      }
-    } else if (n_pv != n_qk) {
-      bool go = ready(&sm.v_full[cv.slot], cv.par);
-      if (go && cv.fresh) {
-        // the first P V of a work item overwrites O: the epilogue of the last item with a tile must have read it
-        go = n_acc == 0 || ready(&sm.o_free[s], (n_acc - 1) & 1);
-        if (go) { cv.fresh = false; started = 0; ++n_acc; }
-      }
-      const uint32_t x = n_pv & 1;
-      if (go) {
-        // with both buffers in use and the next K at hand there is nothing else to do: sleep on it
-        if (n_qk - n_pv == 2 && (k_here || k_end)) {
-          go = __all_sync(full, mbar_wait(&sm.p_full[s][x], (n_pv >> 1) & 1, &sm.abort_flag, wait_limit));
-          if (!go) { ok = false; break; }
-        } else {
-          go = ready(&sm.p_full[s][x], (n_pv >> 1) & 1);
-        }
-      }
-      if (go) {
+        fresh = false;
+        const uint32_t x = n & 1;
+        NEED(&sm.p_full[s][x], (n >> 1) & 1)
         tc_fence_after();
-        const uint32_t v_lo = v_lo0 + cv.slot * (kTileBytes >> 4);
+        const uint32_t v_lo = v_lo0 + slot * (kTileBytes >> 4);
         // lanes of a query block that does not use the tile are left alone; a block's first tile overwrites
-        const uint32_t first = cv.use & ~started, more = cv.use & started;
+        const uint32_t first = use & ~started, more = use & started;
         const uint32_t a_p0 = t_s0 + x * kBlk;
 #pragma unroll
         for (int ks = 0; ks < kBlk / 16; ++ks) {
@@ -624,37 +593,25 @@ __device__ void mma_role(Shared<C>& sm, const Params& p, unsigned char* sQ, unsi
           if (first && leader)
             mma_ts_lanes(t_o, a_p0 + ks * 8, dv, idesc_pv, ks > 0, (first & 1) ? 0u : ~0u, (first & 2) ? 0u : ~0u);
         }
-        started |= cv.use;
+        started |= use;
         if (leader) {
           mma_commit(&sm.pv_done[s][x]);
           // (test hook: a withheld completion signal makes the bounded waits on it run out)
-          if (s != 0 || (int)n_pv != p.withhold_tile) mma_commit(&sm.v_empty[cv.slot]);
+          if (s != 0 || (int)n != p.withhold_tile) mma_commit(&sm.v_empty[slot]);
         }
-        ++n_pv;
-        next_tile(cv);
-        moved = true;
+        ++n;
+      } else if (leader) {
+        mbar_arrive(&sm.v_empty[slot]);
       }
+      if (++slot == kStages) { slot = 0; par ^= 1; }
     }
-    if (moved) {
-      idle = 0;
-    } else if (k_end && !cv.rec && cv.n_rec == ck.n_rec) {
-      break;
-    } else if (idle++ == 0) {
-      t0 = clock64();
-    } else if ((idle & 0x3ffu) == 0) {
-      if (__any_sync(full, *(volatile int*)&sm.abort_flag != 0 || clock64() - t0 > wait_limit)) { ok = false; break; }
-    }
+    if (!ok) break;
+    __syncwarp();
+    if (leader) mbar_arrive(&sm.rec_empty[r]);
   }
-  if (!ok && leader) flag_abort(sm, p, 300 + s);
-  __syncwarp();
-  if (sm.abort_flag) {
-    // Abort path: TMEM must not be released while MMAs are still writing to it, so the role asks for a
-    // completion signal behind everything it has issued and waits for it (bounded).
-    if (leader) mma_commit(&sm.mma_drain[s]);
-    int never = 0;
-    mbar_wait(&sm.mma_drain[s], 0, &never, wait_limit);
-  }
+  drain_mmas(sm, p, ok, leader, 2 + s);
 }
+#undef NEED
 
 // ------------------------------------------------------------------------------------------------
 // softmax + correction + epilogue: one warpgroup of 128 threads per stream; thread = query row.
@@ -860,7 +817,7 @@ __device__ void softmax_role(Shared<C>& sm, const Params& p, uint32_t tmem, int 
 }
 
 template <class C, bool kFromMask>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads64, 1)
 fwd_sm100_b64_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_kc,
                  const __grid_constant__ CUtensorMap tm_vm, const Params p) {
@@ -886,7 +843,7 @@ fwd_sm100_b64_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         mbar_init(&sm.s_full[s][x], 1); mbar_init(&sm.p_full[s][x], 4); mbar_init(&sm.pv_done[s][x], 1);
       }
       mbar_init(&sm.kc_full[s], 1);
-      mbar_init(&sm.mma_drain[s], 1);
+      mbar_init(&sm.mma_drain[s], 1); mbar_init(&sm.mma_drain[2 + s], 1);
     }
     fence_mbar_init();
   }
@@ -907,8 +864,10 @@ fwd_sm100_b64_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     router_role<C, kFromMask>(sm, p, lane);
   } else if (warp == kWarpProducer) {
     if (lane == 0) producer_role<C>(sm, p, sQ, sKV, &tm_q, &tm_k, &tm_v, &tm_kc, &tm_vm);
+  } else if (warp < kWarpPV) {
+    mma_qk_role<C>(sm, p, sQ, sKV, tmem, warp - kWarpQK);
   } else {
-    mma_role<C>(sm, p, sQ, sKV, tmem, warp - kWarpMma);
+    mma_pv_role<C>(sm, p, sKV, tmem, warp - kWarpPV);
   }
   tc_fence_before();
   __syncthreads();
@@ -920,7 +879,7 @@ cudaError_t launch_instance(const Problem& p, const Maps& m, const Params& prm, 
   const size_t smem = 2 * C::kQBytes + 2 * kStages * C::kTileBytes + sizeof(Shared<C>);
   auto kernel = p.routing == SOL_ROUTING_PREPASS && p.mode != SOL_MODE_DENSE ? fwd_sm100_b64_kernel<C, true>
                                                                             : fwd_sm100_b64_kernel<C, false>;
-  return launch_after(kernel, dim3(grid), kThreads, smem, smem, 0, stream, m.q, m.k, m.v, m.kc, m.vm, prm);
+  return launch_after(kernel, dim3(grid), kThreads64, smem, smem, 0, stream, m.q, m.k, m.v, m.kc, m.vm, prm);
 }
 
 }  // namespace
