@@ -2,7 +2,7 @@
 //
 // The tensor core's query tile has 128 rows at full rate (an M = 64 MMA takes as long), so one query block
 // of 64 tokens per tile would leave half of the matrix and softmax work unused.  Here a persistent CTA of
-// 448 threads works on up to 256 consecutive query rows of one head at a time, as two STREAMS of 128 rows,
+// 480 threads works on up to 256 consecutive query rows of one head at a time, as two STREAMS of 128 rows,
 // i.e. four query blocks.  Each stream has its own query tile, score buffers, accumulator, softmax warpgroup
 // and MMA-issuing warp; the two share every K and V tile that both of them need.  The query blocks route
 // independently: a tile is computed for a stream when either of its two blocks wants it, the warps of a
@@ -24,7 +24,7 @@
 //                      (Eq. 4).  The decisions only ever live in a small shared-memory record: a list of
 //                      tile descriptors, each with one flag per query block, and the per-column bias of
 //                      the approximate tile.  Nothing of the proxy map goes to global memory.
-//   producer (warp 9, one lane) reads the records and issues TMA loads: one approximate tile per
+//   producer (warps 9 and 14, one lane each: Q and K; V) reads the records and issues TMA loads: one approximate tile per
 //                      chunk (KC chunk, mean-V chunk) and K_j / V_j ONLY for key blocks that some
 //                      query block of the item routed.
 //   mma      (warps 10-13) two issuing warps per stream, one for the scores and one for P V, with two score
@@ -62,7 +62,8 @@ constexpr int kStages = 4;
 constexpr int kGroup = 16;                       // pooled keys per router staging buffer
 constexpr int kRecords = 4;                      // ring of routing records
 constexpr int kWarpQK = 10, kWarpPV = 12;        // one warp each per stream
-constexpr int kThreads64 = 448;
+constexpr int kWarpProducerV = 14;               // (warp kWarpProducer: query and K tiles)
+constexpr int kThreads64 = 480;
 constexpr int kTmemS = 0, kTmemO = 256;
 
 // Compile-time shape of one kernel instance.
@@ -341,116 +342,95 @@ __device__ void router_role(Shared<C>& sm, const Params& p, int lane) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// producer: one thread.  K and V tiles have rings of their own, and the K loads run up to kLead tiles
-// ahead of the V loads: that is the order in which the slots come free (a K slot when its score
-// GEMMs retire, a V slot a softmax pass and a P V later), so an in-order thread seldom waits for a
-// slot while another load could go.
+// producers: one thread loads the query and K tiles, another (of another warp) the V tiles.  One thread for both needs about
+// 1300 cycles per tile for looking at records and slots in turn and issuing, more than anyone else here: 271 / 260 us at
+// 16 heads x 11 160 tokens, d = 64, keep-or-drop.
+//
+// pooled = true: KC / mean-V operands, dense [B*H][Nk][d]; else q, k, v in the caller's layout.
+// A tile is C::kBoxes boxes of 64 channels, each `box` bytes long in shared memory.
 template <class C>
-__device__ void producer_role(Shared<C>& sm, const Params& p, unsigned char* sQ, unsigned char* sKV,
-                              const CUtensorMap* tm_q, const CUtensorMap* tm_k, const CUtensorMap* tm_v,
-                              const CUtensorMap* tm_kc, const CUtensorMap* tm_vm) {
-  constexpr int kLead = 2;                                   // owed0 and owed1 below
-  constexpr int kTileBytes = C::kTileBytes;
+__device__ __forceinline__ void load_tile(const Params& p, uint32_t bytes, int box, const CUtensorMap* tm, uint64_t* full,
+                                          unsigned char* dst, int row, int b, int h, bool pooled) {
+  mbar_arrive_expect_tx(full, bytes);
+  const bool rows_inner = pooled || p.rows_inner;
+  const int c1 = rows_inner ? row : h, c2 = rows_inner ? h : row;
+  tma_load_4d(dst, tm, full, 0, c1, c2, b);
+  if constexpr (C::kBoxes == 2) tma_load_4d(dst + box, tm, full, 64, c1, c2, b);
+}
+#define NEED(bar, parity) if (!WAIT(bar, parity)) { ok = false; break; }
+
+template <class C>
+__device__ void qk_producer_role(Shared<C>& sm, const Params& p, unsigned char* sQ, unsigned char* sKV,
+                                 const CUtensorMap* tm_q, const CUtensorMap* tm_k, const CUtensorMap* tm_kc) {
   const long long wait_limit = p.wait_limit;
-  uint32_t n_k = 0, n_v = 0, n_rec = 0;
-  uint32_t n_q[2] = {0, 0};
-  // the open record, and the tiles whose V load is still owed (kLead at most, oldest first)
-  const Record* rec = nullptr;
-  int e = 0, end = 0, b = 0, h = 0;
-  uint32_t need_q = 0;
-  struct Tile { uint32_t d; int b, h; } owed0{}, owed1{};
-  // pooled = true: KC / mean-V operands, dense [B*H][Nk][d]; else q, k, v in the caller's layout.
-  // A tile is C::kBoxes boxes of 64 channels, each `box` bytes long in shared memory.
-  auto load_tile = [&](uint32_t bytes, int box, const CUtensorMap* tm, uint64_t* full, unsigned char* dst, int row,
-                       int tb, int th, bool pooled) {
-    mbar_arrive_expect_tx(full, bytes);
-    const bool rows_inner = pooled || p.rows_inner;
-    const int c1 = rows_inner ? row : th, c2 = rows_inner ? th : row;
-    tma_load_4d(dst, tm, full, 0, c1, c2, tb);
-    if constexpr (C::kBoxes == 2) tma_load_4d(dst + box, tm, full, 64, c1, c2, tb);
-  };
-  bool k_end = false, ok = true;
-  for (;;) {
-    // K side (and Q): up to kLead tiles ahead of the V side.  Where a V load is owed, what the K side waits
-    // for may itself wait for that load, so it only looks (test_wait, which never suspends the thread).
-    while (!k_end && (int)(n_k - n_v) < kLead) {
-      if (!rec) {
-        const uint32_t r = n_rec % kRecords, par = (n_rec / kRecords) & 1;
-        if (n_k != n_v && !mbar_test_wait(&sm.rec_full[r], par)) break;
-        if (!WAIT(&sm.rec_full[r], par)) { ok = false; break; }
-        if (sm.rec[r].work < 0) { k_end = true; break; }
-        rec = &sm.rec[r];
-        e = 0;
-        end = rec->n;
-        b = rec->b;
-        h = rec->h;
-        need_q = 0;
-        if (rec->flags & kRecFirst) need_q = (rec->valid & 1) | ((rec->valid >> kSub) & 1) << 1;
-      }
+  uint32_t n = 0, n_q[2] = {0, 0};             // K tiles and query tiles so far
+  bool ok = true;
+  for (uint32_t n_rec = 0; ok; ++n_rec) {
+    const uint32_t r = n_rec % kRecords;
+    NEED(&sm.rec_full[r], (n_rec / kRecords) & 1)
+    const Record& rec = sm.rec[r];
+    if (rec.work < 0) break;
+    const int n_desc = rec.n, b = rec.b, h = rec.h;
+    if (rec.flags & kRecFirst) {
       // Q of both streams, once per work item.  A slot frees when the stream's last score GEMM of the
       // previous item retires.
-      if (need_q) {
-        bool busy = false;
 #pragma unroll
-        for (int s = 0; s < 2; ++s) {
-          if (!((need_q >> s) & 1)) continue;
-          const uint32_t par = (n_q[s] & 1) ^ 1;
-          if (n_k != n_v && !mbar_test_wait(&sm.q_empty[s], par)) { busy = true; continue; }
-          if (!WAIT(&sm.q_empty[s], par)) { ok = false; break; }
-          load_tile(C::kQBytes, C::kQBoxBytes, tm_q, &sm.q_full[s], sQ + s * C::kQBytes, rec->q_row[s], b, h, false);
-          ++n_q[s];
-          need_q &= ~(1u << s);
-        }
-        if (!ok || busy) break;
+      for (int s = 0; s < 2; ++s) {
+        if (!((rec.valid >> (s * kSub)) & 1)) continue;
+        NEED(&sm.q_empty[s], (n_q[s] & 1) ^ 1)
+        load_tile<C>(p, C::kQBytes, C::kQBoxBytes, tm_q, &sm.q_full[s], sQ + s * C::kQBytes, rec.q_row[s], b, h, false);
+        ++n_q[s];
       }
-      if (e < end) {
-        const uint32_t d = rec->desc[e];
-        const uint32_t s = n_k % kStages;
-        if (!WAIT(&sm.k_empty[s], ((n_k / kStages) & 1) ^ 1)) { ok = false; break; }
-        load_tile(kTileBytes, C::kBoxBytes, (d & kTileApprox) ? tm_kc : tm_k, &sm.k_full[s],
-                  sKV + (size_t)s * kTileBytes, (int)(d >> 5), b, h, (d & kTileApprox) != 0);
-        if (n_k == n_v) owed0 = Tile{d, b, h};
-        else owed1 = Tile{d, b, h};
-        ++n_k;
-        ++e;
-      }
-      if (e == end) {
-        mbar_arrive(&sm.rec_empty[n_rec % kRecords]);
-        rec = nullptr;
-        ++n_rec;
-      }
+      if (!ok) break;
     }
-    if (!ok) break;
-    if (n_k == n_v) {
-      if (k_end) break;
-      continue;
+    for (int e = 0; e < n_desc; ++e, ++n) {
+      const uint32_t d = rec.desc[e], s = n % kStages;
+      NEED(&sm.k_empty[s], ((n / kStages) & 1) ^ 1)
+      load_tile<C>(p, C::kTileBytes, C::kBoxBytes, (d & kTileApprox) ? tm_kc : tm_k, &sm.k_full[s],
+                   sKV + (size_t)s * C::kTileBytes, (int)(d >> 5), b, h, (d & kTileApprox) != 0);
     }
-    // V side: the oldest tile whose K is already on its way
-    const uint32_t s = n_v % kStages;
-    const Tile t = owed0;
-    owed0 = owed1;
-    if (!WAIT(&sm.v_empty[s], ((n_v / kStages) & 1) ^ 1)) { ok = false; break; }
-    load_tile(kTileBytes, C::kBoxBytes, (t.d & kTileApprox) ? tm_vm : tm_v, &sm.v_full[s],
-              sKV + (size_t)(kStages + s) * kTileBytes, (int)(t.d >> 5), t.b, t.h, (t.d & kTileApprox) != 0);
-    ++n_v;
+    if (ok) mbar_arrive(&sm.rec_empty[r]);
   }
   if (!ok) flag_abort(sm, p, 200);
   // The consumers wait for every K, V and Q tile of a normal run; after an abort, let copies that are
   // still in flight land before the CTA's shared memory goes away.
   if (sm.abort_flag) {
-    int never = 0;                                   // this drain must not be cut short by the abort flag
+    int never = 0;                             // this drain must not be cut short by the abort flag
     for (int s = 0; s < 2; ++s)
       if (n_q[s] > 0) mbar_wait(&sm.q_full[s], (n_q[s] - 1) & 1, &never, wait_limit);
-    for (uint32_t back = 0; back < kStages && back < n_k; ++back) {
-      const uint32_t n = n_k - 1 - back;
-      mbar_wait(&sm.k_full[n % kStages], (n / kStages) & 1, &never, wait_limit);
-    }
-    for (uint32_t back = 0; back < kStages && back < n_v; ++back) {
-      const uint32_t n = n_v - 1 - back;
-      mbar_wait(&sm.v_full[n % kStages], (n / kStages) & 1, &never, wait_limit);
-    }
+    for (uint32_t back = 1; back <= kStages && back <= n; ++back)
+      mbar_wait(&sm.k_full[(n - back) % kStages], ((n - back) / kStages) & 1, &never, wait_limit);
   }
 }
+
+template <class C>
+__device__ void v_producer_role(Shared<C>& sm, const Params& p, unsigned char* sKV, const CUtensorMap* tm_v,
+                                const CUtensorMap* tm_vm) {
+  const long long wait_limit = p.wait_limit;
+  uint32_t n = 0;
+  bool ok = true;
+  for (uint32_t n_rec = 0; ok; ++n_rec) {
+    const uint32_t r = n_rec % kRecords;
+    NEED(&sm.rec_full[r], (n_rec / kRecords) & 1)
+    const Record& rec = sm.rec[r];
+    if (rec.work < 0) break;
+    const int n_desc = rec.n, b = rec.b, h = rec.h;
+    for (int e = 0; e < n_desc; ++e, ++n) {
+      const uint32_t d = rec.desc[e], s = n % kStages;
+      NEED(&sm.v_empty[s], ((n / kStages) & 1) ^ 1)
+      load_tile<C>(p, C::kTileBytes, C::kBoxBytes, (d & kTileApprox) ? tm_vm : tm_v, &sm.v_full[s],
+                   sKV + (size_t)(kStages + s) * C::kTileBytes, (int)(d >> 5), b, h, (d & kTileApprox) != 0);
+    }
+    if (ok) mbar_arrive(&sm.rec_empty[r]);
+  }
+  if (!ok) flag_abort(sm, p, 201);
+  if (sm.abort_flag) {
+    int never = 0;
+    for (uint32_t back = 1; back <= kStages && back <= n; ++back)
+      mbar_wait(&sm.v_full[(n - back) % kStages], ((n - back) / kStages) & 1, &never, wait_limit);
+  }
+}
+#undef NEED
 
 // ------------------------------------------------------------------------------------------------
 // Two issuing warps per stream s, one for the score GEMMs and one for the value GEMMs.  A warp that did both had to look at
@@ -830,8 +810,8 @@ fwd_sm100_b64_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
 
   if (threadIdx.x == 0) {
     sm.abort_flag = 0;
-    // a record is released by the producer, the two MMA warps' two cursors and the 8 softmax warps
-    for (int r = 0; r < kRecords; ++r) { mbar_init(&sm.rec_full[r], 1); mbar_init(&sm.rec_empty[r], 13); }
+    // a record is released by the two producers, the four MMA warps and the 8 softmax warps
+    for (int r = 0; r < kRecords; ++r) { mbar_init(&sm.rec_full[r], 1); mbar_init(&sm.rec_empty[r], 14); }
     for (int i = 0; i < kStages; ++i) {                      // a tile is released by both MMA warps
       mbar_init(&sm.k_full[i], 1); mbar_init(&sm.k_empty[i], 2);
       mbar_init(&sm.v_full[i], 1); mbar_init(&sm.v_empty[i], 2);
@@ -863,7 +843,9 @@ fwd_sm100_b64_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
   } else if (warp == kWarpRouter) {
     router_role<C, kFromMask>(sm, p, lane);
   } else if (warp == kWarpProducer) {
-    if (lane == 0) producer_role<C>(sm, p, sQ, sKV, &tm_q, &tm_k, &tm_v, &tm_kc, &tm_vm);
+    if (lane == 0) qk_producer_role<C>(sm, p, sQ, sKV, &tm_q, &tm_k, &tm_kc);
+  } else if (warp == kWarpProducerV) {
+    if (lane == 0) v_producer_role<C>(sm, p, sKV, &tm_v, &tm_vm);
   } else if (warp < kWarpPV) {
     mma_qk_role<C>(sm, p, sQ, sKV, tmem, warp - kWarpQK);
   } else {
