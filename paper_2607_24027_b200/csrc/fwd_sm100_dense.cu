@@ -376,8 +376,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 fwd_sm100_dense_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                        const __grid_constant__ CUtensorMap tm_v, const Params p, int block) {
   using C = Cfg<D>;
-  extern __shared__ __align__(1024) unsigned char smem_raw[];   // (see fwd_sm100.cu)
-  unsigned char* sQ = smem_raw;
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* sQ = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   unsigned char* sKV = sQ + 2 * C::kTileBytes;
   Shared& sm = *reinterpret_cast<Shared*>(sKV + kSlots * C::kTileBytes);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -427,7 +427,7 @@ cudaError_t launch_instance(const Problem& p, const Maps& m, const Params& prm, 
     if (a.numRegs < kRegsLaunch) return cudaErrorInvalidConfiguration;
     enough = true;
   }
-  const size_t smem = (2 + kSlots) * Cfg<D>::kTileBytes + sizeof(Shared);
+  const size_t smem = 1024 + (2 + kSlots) * Cfg<D>::kTileBytes + sizeof(Shared);
   return launch_after(fwd_sm100_dense_kernel<D>, dim3(grid), kThreads, smem, smem, 0, stream, m.q, m.k, m.v, prm, p.block_q);
 }
 
