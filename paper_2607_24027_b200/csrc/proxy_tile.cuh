@@ -1,5 +1,5 @@
-// fp32 product of pooled queries and pooled keys, one 128 x 64 tile per CTA, left in registers: what the routing
-// pre-pass (decision bits) and the materialised baselines (the proxy map) both start from.
+// fp32 product of pooled queries and pooled keys, one 128 x 64 tile per CTA, left in registers: what the materialised
+// baselines write out as the proxy map.  (The routing pre-pass forms its products on the tensor core, route_prepass.cu.)
 #pragma once
 
 #include <cuda_runtime.h>
