@@ -54,7 +54,7 @@ struct Problem {
 //     3918 / 3695.
 //   64-token blocks: up to one block per SM fwd_sm100.cu (2 x 4096 tokens, d = 128: 55 / 68).  Above that the other kernel,
 //     fwd_sm100_b64.cu, also takes 256 rows at a time, but tiles of 64 keys; pairs take 0.74 to 0.85 of its time up to
-//     40 x 16 000 tokens.
+//     40 x 16 000 tokens (taken before its roles were split, which took 15 to 18 % off it in the routed modes).
 inline bool dense_in_pairs(int BH, int N, int d, int block_k, int sms) {
   if (block_k == 64) return (long long)BH * ceil_div(N, 64) > sms;
   const long long tiles = (long long)BH * ceil_div(N, 128), pairs = (long long)BH * ceil_div(N, 256);
