@@ -17,12 +17,18 @@ using namespace ptx;
 
 // The products are those of fp32 numbers: each is cut into three bf16 parts, x = x1 + x2 + x3 (8 significant bits each, so the
 // sum is x), and of the nine products of parts the six that matter in fp32 are formed by the tensor core,
-//   x y = x1 y1 + (x1 y2 + x2 y1 + x2 y2 + x1 y3 + x3 y1),   the rest below 2^-26 of |x| |y|.
+//   x y = x1 y1 + (x1 y2 + x2 y1 + x2 y2 + x1 y3 + x3 y1),   the rest 2^-24 of |x| |y| at the most, 2^-27 as a rule.
 // Products of bf16 parts are exact in fp32.  The small terms have an accumulator of their own, so that they are not
 // rounded at the size of the large ones, and the first term has two: the tensor core rounds towards zero when it adds, and
 // every addition counts.  Error of the scores against 64 bits, relative 2-norm (packed FMAs of proxy_tile.cuh / this with one, two,
 // three accumulators of the first term), d = 128: 40 x 591 x 591 blocks 1.44e-7 / - / 1.31e-7 / 1.11e-7, 24 x 32 x 32
 // 1.53e-7 / 2.81e-7 / 1.35e-7 / 1.32e-7; d = 64, 16 x 175 x 175 1.06e-7 / 1.09e-7 / 0.72e-7 / 0.69e-7.
+//
+// What this cannot form is formed with FMAs instead, in the order in which proxy_tile.cuh forms it (`direct_score`):
+//   - a tile with an infinity, a NaN or a number from 2^60 on.  The first two have no parts.  Where products leave the range of
+//     fp32, parts of both signs make a NaN of what the FMAs make an infinity (x = y = 1.0039 * 2^64: x1 y1 = inf, x1 y2 = -inf),
+//     and the tensor core, which adds 16 products before it rounds, may see no overflow at all;
+//   - a tile with a number below 2^-50 that is not zero, whose parts' products can be too small for fp32 to hold.
 //
 // 40 heads x 591 x 591 blocks, d = 128: 113 us with packed FMAs on the CUDA cores, 37 us so (two accumulators; 128 x 64 tiles
 // 49 us).  Its floor is the tensor core's: 1000 tiles of 48 MMAs, 13 us; the rest is cutting (a third of the instructions) and
@@ -56,8 +62,27 @@ __device__ __forceinline__ Parts split(float4 v) {
   }
   return r;
 }
-__device__ __forceinline__ bool not_finite(float4 v) {
-  return !(fabsf(v.x) < INFINITY && fabsf(v.y) < INFINITY && fabsf(v.z) < INFINITY && fabsf(v.w) < INFINITY);
+// Smallest and largest magnitude of the numbers seen so far, by their first parts (in 16-bit halves).  `least` is one less than
+// that: zero less one is the largest number there is, so that zeros do not count.
+struct Range {
+  uint32_t least = 0xffffffffu, most = 0;
+  __device__ __forceinline__ void add(uint2 parts) {
+    const uint32_t a = parts.x & 0x7fff7fffu, b = parts.y & 0x7fff7fffu;
+    least = __viaddmin_u16x2(b, 0xffffffffu, __viaddmin_u16x2(a, 0xffffffffu, least));
+    most = __vimax3_u16x2(a, b, most);
+  }
+  __device__ __forceinline__ bool left() const {
+    return min(least & 0xffffu, least >> 16) + 1 < (127 - 50) << 7 || max(most & 0xffffu, most >> 16) >= (127 + 60) << 7;
+  }
+};
+
+__device__ __noinline__ float direct_score(const float* __restrict__ q, const float* __restrict__ k, int d) {
+  float even = 0.f, odd = 0.f;
+  for (int c = 0; c < d; c += 2) {
+    even = fmaf(q[c], k[c], even);
+    odd = fmaf(q[c + 1], k[c + 1], odd);
+  }
+  return even + odd;
 }
 
 // grid (ceil(Nk / 128), ceil(Nq / 128), BH).  mask[bh][i][w]: bit j % 32 of word j / 32 = block j routed.
@@ -81,7 +106,8 @@ mask_prepass_kernel(const float* __restrict__ qbar, const float* __restrict__ kc
   const uint32_t lo0 = (smem_addr(parts) >> 4) | (1u << 16);
   int never = 0;
   uint32_t tmem = 0;
-  bool ok = true, special = false;
+  Range range;
+  bool ok = true;
   for (int c0 = 0, chunk = 0; c0 < d; c0 += kChunk, ++chunk) {
     // 16 threads per row, 16 rows at a time: query blocks, then key blocks
     const int c4 = tid % 16;
@@ -98,7 +124,7 @@ mask_prepass_kernel(const float* __restrict__ qbar, const float* __restrict__ kc
     for (int x = 0; x < kQ + kK; ++x) {
       const int r = tid / 16 + 16 * (x < kQ ? x : x - kQ);     // below 128 or kKeys: the row stays inside its part
       const Parts s = split(v[x]);
-      special |= not_finite(v[x]);
+      range.add(s.p[0]);
       unsigned char* dst = parts + (x < kQ ? 0 : 3 * kPartBytes) + r * 128 + (((c4 / 2) ^ (r & 7)) * 16) + (c4 & 1) * 8;
 #pragma unroll
       for (int part = 0; part < 3; ++part) *reinterpret_cast<uint2*>(dst + part * (x < kQ ? kPartBytes : kKeyPartBytes)) = s.p[part];
@@ -130,8 +156,8 @@ mask_prepass_kernel(const float* __restrict__ qbar, const float* __restrict__ kc
   }
   if (ok) ok = mbar_wait(&done, (ceil_div(d, kChunk) - 1) & 1, &never);
   tc_fence_after();
-  special = __syncthreads_or(special);
   ok = __syncthreads_and(ok);
+  const bool direct = __syncthreads_or(range.left() || !ok);
   // thread = query block, half of the key blocks each
   const int row = (warp % 4) * 32 + lane, col0 = (warp / 4) * (kKeys / 2);
   const int i = i0 + row, words = ceil_div(Nk, 32);
@@ -140,7 +166,7 @@ mask_prepass_kernel(const float* __restrict__ qbar, const float* __restrict__ kc
   for (int c = 0; c < kKeys / 64; ++c) {
     const int j = j0 + col0 + 32 * c;            // this word's first key block
     uint32_t word = 0;
-    if (!special && ok) {
+    if (!direct) {
       uint32_t acc[kMains + 1][32];
 #pragma unroll
       for (int x = 0; x <= kMains; ++x)
@@ -154,13 +180,12 @@ mask_prepass_kernel(const float* __restrict__ qbar, const float* __restrict__ kc
         word |= (scale * dot > t ? 1u : 0u) << b;
       }
     } else if (ok && row < nq) {
-      // infinities and NaN have no parts: the products as they are
       for (int b = 0; b < 32 && j + b < Nk; ++b) {
-        float dot = 0.f;
-        for (int x = 0; x < d; ++x) dot = fmaf(q[(size_t)row * d + x], k[(size_t)(j - j0 + b) * d + x], dot);
+        const float dot = direct_score(q + (size_t)row * d, k + (size_t)(j - j0 + b) * d, d);
         word |= (scale * dot > t ? 1u : 0u) << b;
       }
     }
+    __syncwarp();
     word |= __ballot_sync(0xffffffffu, forced && j + lane < Nk && forced[j + lane]);
     if (j + 32 > Nk) word &= j < Nk ? (1u << (Nk - j)) - 1u : 0u;
     if (i < Nq && j < Nk) mask[((size_t)bh * Nq + i) * words + j / 32] = word;
