@@ -155,7 +155,9 @@ sol_status_t sol_attn_dense(const void* q, const void* k, const void* v, void* o
  * sol_attn_thresholds / forward left in the bound workspace, and writes one bit per pair to `mask`
  * (device, uint32 [B, H, Nq, ceil(Nk / 32)], bit j % 32 of word j / 32; caller-owned).  `tau_override`
  * (device fp32 [B, H, Nq]) replaces the workspace's thresholds when not NULL; `forced_blocks` as in
- * sol_attn_args.  `scale` <= 0 selects 1/sqrt(d).  One kernel on `stream`; does not synchronise. */
+ * sol_attn_args.  `scale` <= 0 selects 1/sqrt(d).  One kernel on `stream`; does not synchronise.  Reports nothing
+ * in the status word and does not touch it: bits whose tensor-core products do not arrive within the wait limit
+ * are formed on the CUDA cores instead. */
 sol_status_t sol_attn_route_mask(int B, int H, int N, int d, int block_q, int block_k, float scale,
                                  const float* tau_override, const uint8_t* forced_blocks, uint32_t* mask,
                                  sol_stream_t stream);
@@ -224,7 +226,9 @@ sol_status_t sol_attn_forward_host(const void* hq, const void* hk, const void* h
                                    float threshold, sol_stream_t stream);
 
 /* Synchronises `stream`, then returns the device status word of the bound workspace
- * (SOL_OK, or SOL_ERR_DEVICE_TIMEOUT when a kernel gave up on a bounded wait) and clears it. */
+ * (SOL_OK, or SOL_ERR_DEVICE_TIMEOUT when a kernel gave up on a bounded wait) and clears it.
+ * A forward sets the word anew; sol_attn_pool, sol_attn_thresholds and sol_attn_route_mask have no such
+ * error and leave it alone, so a workspace that no forward has used yet holds no status. */
 sol_status_t sol_attn_read_device_status(sol_stream_t stream);
 
 /* Threshold step for callers that cannot allocate device memory.  (The paper has no counterpart:
@@ -295,6 +299,8 @@ int64_t sol_attn_launch_count(void);
  * whose "value GEMM finished" signal is left out (withhold_tile < 0: none).  With a tile withheld the
  * waits on that signal run out, every warp role drains, TMEM is released, the kernel returns and
  * sol_attn_read_device_status() reports SOL_ERR_DEVICE_TIMEOUT; the outputs of that launch are invalid.
+ * In the routing-bits kernel the index is that of 64 channels whose "products finished" signal is left out; its
+ * bits stay right (see sol_attn_route_mask).
  * Nothing faults, traps or spins without a bound.  Not for production use; not thread-safe. */
 void sol_attn_debug_set_wait(int64_t wait_cycles, int32_t withhold_tile);
 

@@ -655,10 +655,6 @@ fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 }
 
-// Test hook (sol_attn_debug_set_wait): the wait limit and the withheld tile of the following launches.
-long long g_wait_limit = kWaitCycles;
-int g_withhold_tile = -1;
-
 template <class C>
 cudaError_t launch_instance(const Problem& p, const Maps& m, const Params& prm, int grid, cudaStream_t stream) {
   const size_t smem = C::kQBytes + (kKStages + kVStages) * C::kTileBytes + sizeof(Shared<C>);
@@ -668,6 +664,10 @@ cudaError_t launch_instance(const Problem& p, const Maps& m, const Params& prm, 
 }
 
 }  // namespace
+
+long long g_wait_limit = kWaitCycles;
+int g_withhold_tile = -1;
+
 }  // namespace fwd
 
 bool fwd_sm100_supports(const Problem& p) {

@@ -36,6 +36,10 @@ struct Params {
   int per_item, items_per_head; // 64-token blocks: query blocks per work item
 };
 
+// Test hook (sol_attn_debug_set_wait): the wait limit and the withheld tile of the following launches (fwd_sm100.cu).
+extern long long g_wait_limit;
+extern int g_withhold_tile;
+
 struct Maps {                   // q, k, v in the caller's layout; KC and mean-V, dense [B][H][Nk][d]
   CUtensorMap q, k, v, kc, vm;
 };

@@ -28,20 +28,29 @@ using namespace ptx;
 //   - a tile with an infinity, a NaN or a number from 2^60 on.  The first two have no parts.  Where products leave the range of
 //     fp32, parts of both signs make a NaN of what the FMAs make an infinity (x = y = 1.0039 * 2^64: x1 y1 = inf, x1 y2 = -inf),
 //     and the tensor core, which adds 16 products before it rounds, may see no overflow at all;
-//   - a tile with a number below 2^-50 that is not zero, whose parts' products can be too small for fp32 to hold.
+//   - a tile with a number below 2^-50 that is not zero, whose parts' products can be too small for fp32 to hold;
+//   - a tile whose MMAs did not retire within the wait limit.  So the bits are right in that case too, and this
+//     kernel has no error to report.
 //
-// 40 heads x 591 x 591 blocks, d = 128: 113 us with packed FMAs on the CUDA cores, 37 us so (two accumulators; 128 x 64 tiles
-// 49 us).  Its floor is the tensor core's: 1000 tiles of 48 MMAs, 13 us; the rest is cutting (a third of the instructions) and
-// the comparison, which two CTAs per SM overlap with the other's MMAs in part.
+// 40 heads x 591 x 591 blocks, d = 128: 113 us with packed FMAs on the CUDA cores, 35 us so (two accumulators; 128 x 64 tiles
+// 49 us; 0.7 us for looking at the range of the numbers); 24 x 32 x 32 blocks 10.3 / 6.4 us.  Its floor is the tensor core's: 1000
+// tiles of 48 MMAs, 13 us; the rest is cutting (a third of the instructions) and the comparison, which two CTAs per SM
+// overlap with the other's MMAs in part.
 constexpr int kTile = 128;                       // query blocks per CTA
 constexpr int kKeys = 128;                       // key blocks per CTA
 constexpr int kChunk = 64;                       // channels in shared memory at a time
 constexpr int kPartBytes = kTile * kChunk * 2;   // one bf16 part of one operand: a 128-byte row per block, 128-byte swizzle
 constexpr int kThreadsMask = 256;
 constexpr int kKeyPartBytes = kKeys * kChunk * 2;
-constexpr size_t kMaskSmem = 1024 + 3 * (kPartBytes + kKeyPartBytes);
 constexpr int kMains = 2;                        // accumulators of the first term
 constexpr int kMaskCols = 512;                   // tensor-memory columns: kMains + 1 accumulators of kKeys, a power of two
+
+struct MaskShared {                              // behind the parts
+  uint64_t done;                                 // the MMAs of a chunk have retired
+  uint64_t drain;                                // a wait for that ran out: all MMAs issued have retired
+  uint32_t tmem;
+};
+constexpr size_t kMaskSmem = 3 * (kPartBytes + kKeyPartBytes) + sizeof(MaskShared);
 
 struct Parts { uint2 p[3]; };                    // four channels: three parts of bf16
 
@@ -88,15 +97,14 @@ __device__ __noinline__ float direct_score(const float* __restrict__ q, const fl
 // grid (ceil(Nk / 128), ceil(Nq / 128), BH).  mask[bh][i][w]: bit j % 32 of word j / 32 = block j routed.
 __global__ void __launch_bounds__(kThreadsMask, 2)
 mask_prepass_kernel(const float* __restrict__ qbar, const float* __restrict__ kc, const float* __restrict__ tau,
-                    const uint8_t* __restrict__ forced, uint32_t* __restrict__ mask, int32_t* __restrict__ status, int Nq, int Nk,
-                    int d, float scale) {
+                    const uint8_t* __restrict__ forced, uint32_t* __restrict__ mask, int Nq, int Nk, int d, float scale,
+                    long long wait_limit, int withhold) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  __shared__ uint64_t done;                      // the MMAs of a chunk have retired
-  __shared__ uint32_t tmem_s;
-  unsigned char* parts = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  unsigned char* parts = smem_raw;
+  MaskShared& sm = *reinterpret_cast<MaskShared*>(smem_raw + 3 * (kPartBytes + kKeyPartBytes));
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   const int bh = blockIdx.z, i0 = blockIdx.y * kTile, j0 = blockIdx.x * kKeys;
-  if (tid == 0) { mbar_init(&done, 1); fence_mbar_init(); }
+  if (tid == 0) { mbar_init(&sm.done, 1); mbar_init(&sm.drain, 1); fence_mbar_init(); }
   __syncthreads();
   kernel_wait();
   const float* q = qbar + ((size_t)bh * Nq + i0) * d;
@@ -104,10 +112,11 @@ mask_prepass_kernel(const float* __restrict__ qbar, const float* __restrict__ kc
   const int nq = min(kTile, Nq - i0), nk = min(kKeys, Nk - j0);
   const uint32_t idesc = make_idesc_bf16(kTile, kKeys, false, false);
   const uint32_t lo0 = (smem_addr(parts) >> 4) | (1u << 16);
+  const bool leader = warp == 0 && elect_one();  // issues all MMAs and their completion signals
   int never = 0;
   uint32_t tmem = 0;
   Range range;
-  bool ok = true;
+  bool ok = true;                                // no wait has run out
   for (int c0 = 0, chunk = 0; c0 < d; c0 += kChunk, ++chunk) {
     // 16 threads per row, 16 rows at a time: query blocks, then key blocks
     const int c4 = tid % 16;
@@ -119,7 +128,7 @@ mask_prepass_kernel(const float* __restrict__ qbar, const float* __restrict__ kc
       v[x] = r < (x < kQ ? nq : nk) ? __ldg(reinterpret_cast<const float4*>((x < kQ ? q : k) + (size_t)r * d + c0) + c4)
                                     : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    if (chunk > 0 && ok) ok = mbar_wait(&done, (chunk - 1) & 1, &never);   // the parts of the chunk before have been read
+    if (chunk > 0) ok = mbar_wait(&sm.done, (chunk - 1) & 1, &never, wait_limit);   // the parts of the chunk before have been read
 #pragma unroll
     for (int x = 0; x < kQ + kK; ++x) {
       const int r = tid / 16 + 16 * (x < kQ ? x : x - kQ);     // below 128 or kKeys: the row stays inside its part
@@ -132,13 +141,13 @@ mask_prepass_kernel(const float* __restrict__ qbar, const float* __restrict__ kc
     fence_proxy_async_smem();
     if (chunk == 0) {
       // this late, so that of two CTAs on an SM one loads and cuts while the other has the tensor memory
-      if (warp == 0) { tmem_alloc(&tmem_s, kMaskCols); tmem_relinquish(); }
+      if (warp == 0) { tmem_alloc(&sm.tmem, kMaskCols); tmem_relinquish(); }
       tc_fence_before();
     }
-    __syncthreads();
-    tmem = *const_cast<volatile uint32_t*>(&tmem_s);
+    ok = __syncthreads_and(ok);
+    tmem = *const_cast<volatile uint32_t*>(&sm.tmem);
+    if (!ok) break;                              // (a wait ran out: not in the first chunk)
     if (warp == 0) {
-      const bool leader = elect_one();
       tc_fence_after();
       constexpr int kP[6][2] = {{0, 1}, {1, 0}, {1, 1}, {0, 2}, {2, 0}, {0, 0}};   // the first term comes last
 #pragma unroll
@@ -150,11 +159,12 @@ mask_prepass_kernel(const float* __restrict__ qbar, const float* __restrict__ kc
           const bool fresh = chunk == 0 && (t == 5 ? ks < kMains : (t == 0 && ks == 0));
           if (leader) mma_ss(tmem + acc * kKeys, fwd::desc_from_lo(a), fwd::desc_from_lo(b), idesc, fresh ? 0u : 1u);
         }
-      if (leader) mma_commit(&done);
+      // (test hook: a withheld completion signal makes the waits on it run out)
+      if (leader && chunk != withhold) mma_commit(&sm.done);
     }
     __syncwarp();
   }
-  if (ok) ok = mbar_wait(&done, (ceil_div(d, kChunk) - 1) & 1, &never);
+  if (ok) ok = mbar_wait(&sm.done, (ceil_div(d, kChunk) - 1) & 1, &never, wait_limit);
   tc_fence_after();
   ok = __syncthreads_and(ok);
   const bool direct = __syncthreads_or(range.left() || !ok);
@@ -179,7 +189,7 @@ mask_prepass_kernel(const float* __restrict__ qbar, const float* __restrict__ kc
         for (int x = 1; x <= kMains; ++x) dot += __uint_as_float(acc[x][b]);
         word |= (scale * dot > t ? 1u : 0u) << b;
       }
-    } else if (ok && row < nq) {
+    } else if (row < nq) {
       for (int b = 0; b < 32 && j + b < Nk; ++b) {
         const float dot = direct_score(q + (size_t)row * d, k + (size_t)(j - j0 + b) * d, d);
         word |= (scale * dot > t ? 1u : 0u) << b;
@@ -190,9 +200,10 @@ mask_prepass_kernel(const float* __restrict__ qbar, const float* __restrict__ kc
     if (j + 32 > Nk) word &= j < Nk ? (1u << (Nk - j)) - 1u : 0u;
     if (i < Nq && j < Nk) mask[((size_t)bh * Nq + i) * words + j / 32] = word;
   }
-  if (!ok && tid == 0) {
-    atomicExch(status + kStatusDevice, (int)SOL_ERR_DEVICE_TIMEOUT);
-    atomicCAS(status + kStatusDetail, 0, 500);
+  if (warp == 0 && !ok) {
+    // the tensor memory must not be released while MMAs still write to it: wait (bounded) behind all that were issued
+    if (leader) mma_commit(&sm.drain);
+    mbar_wait(&sm.drain, 0, &never, wait_limit);
   }
   tc_fence_before();
   __syncthreads();
@@ -206,7 +217,7 @@ cudaError_t launch_route_prepass(const Problem& p, const WsPtrs& ws, const float
   const dim3 grid(ceil_div(p.Nk, kKeys), ceil_div(p.Nq, kTile), p.BH);
   if (n_launches) *n_launches += 1;
   return launch_after(mask_prepass_kernel, grid, kThreadsMask, kMaskSmem, kMaskSmem, 0, stream, ws.qbar, ws.kc, tau, p.forced,
-                      mask, ws.status, p.Nq, p.Nk, p.d, p.scale);
+                      mask, p.Nq, p.Nk, p.d, p.scale, fwd::g_wait_limit, fwd::g_withhold_tile);
 }
 
 }  // namespace sol

@@ -65,10 +65,12 @@ def _bits(q, k, tau):
     N = nq * 64
     ws = sb.make_workspace(1, heads, N, d, 64, 64)
     sb.sol_attn_bind_workspace(ws)
+    ws.buf[:64].fill_(90)                          # the status words, which are not this call's
     ws.qbar.copy_(torch.from_numpy(q)), ws.kc.copy_(torch.from_numpy(k))
     mask = torch.full((1, heads, nq, sb.mask_words(nq)), -1, dtype=torch.int32, device="cuda")
     tau = torch.from_numpy(np.ascontiguousarray(tau))[None].cuda()
     sb.sol_attn_route_mask(1, heads, N, d, 64, 64, mask, scale=1.0, tau_override=tau)
+    assert bool((ws.buf[:64] == 90).all())
     bits = (mask[0].long()[..., None] >> torch.arange(32, device="cuda")) & 1
     return bits.flatten(-2).bool()[..., :nq].cpu().numpy()
 
@@ -130,3 +132,21 @@ def test_scores_beyond_fp32(n, d):
     near = (np.abs(s.astype(np.float64) - tau[:, :, None]) <= 2 * math.sqrt(d) * 2.0 ** -24 * size) & np.isfinite(s)
     assert not near[~np.isfinite(s)].any() and near.mean() < 0.5
     assert bool(((_bits(q, k, tau) == (s > tau[:, :, None])) | near).all())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,d,withhold", [(129, 64, 0), (129, 128, 0), (129, 128, 1)])
+def test_without_a_completion_signal(n, d, withhold):
+    """The wait for the tensor core runs out after about a millisecond: the bits come from FMAs, the tensor memory goes back
+    behind the MMAs, and the next call is a normal one."""
+    from paper_2607_24027_b200 import binding as sb
+    q, k, tau, s, near = _one_product(2, n, n, d, n + d)
+    want = s > tau[:, :, None]
+    sb.sol_attn_debug_set_wait(2_000_000, withhold)
+    try:
+        bits = _bits(q, k, tau)
+        torch.cuda.synchronize()
+    finally:
+        sb.sol_attn_debug_set_wait(0, -1)
+    assert bool(((bits == want) | near).all())
+    assert bool(((_bits(q, k, tau) == want) | near).all())
