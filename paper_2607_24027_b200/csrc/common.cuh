@@ -52,9 +52,10 @@ struct Problem {
 //     24 x 8500 (11 / 6) 869 / 890; 40 x 8192 (18 / 9) 1341 / 1304.
 //     d = 64: 12 x 4096 (3 / 2) 101 / 115; 24 x 4096 (6 / 3) 188 / 169; 30 x 4096 (7 / 4) 221 / 221; 40 x 16 000 (34 / 18)
 //     3918 / 3695.
-//   64-token blocks: up to one block per SM fwd_sm100.cu (2 x 4096 tokens, d = 128: 55 / 68).  Above that the other kernel,
-//     fwd_sm100_b64.cu, also takes 256 rows at a time, but tiles of 64 keys; pairs take 0.74 to 0.85 of its time up to
-//     40 x 16 000 tokens (taken before its roles were split, which took 15 to 18 % off it in the routed modes).
+//   64-token blocks: up to one block per SM fwd_sm100.cu (2 x 4096 tokens, d = 64 50 / 60, d = 128 56 / 68; 148 blocks, d = 64
+//     56 / 69).  Above that always pairs: fwd_sm100_b64.cu, which also takes 256 rows at a time but tiles of 64 keys, has no
+//     dense mode, in which it took 1.03 to 1.18 times as long (150 blocks, d = 64 80 / 70 us; 24 x 4096 tokens 192 / 169;
+//     40 x 16 000 3965 / 3690; d = 128 12 x 4096 140 / 135).
 inline bool dense_in_pairs(int BH, int N, int d, int block_k, int sms) {
   if (block_k == 64) return (long long)BH * ceil_div(N, 64) > sms;
   const long long tiles = (long long)BH * ceil_div(N, 128), pairs = (long long)BH * ceil_div(N, 256);

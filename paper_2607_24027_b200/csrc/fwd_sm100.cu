@@ -693,7 +693,7 @@ cudaError_t launch_fwd_sm100(const Problem& p, const __nv_bfloat16* q, const __n
   // 64-token blocks: several query blocks per CTA need more blocks than SMs.  Up to one block per SM a CTA has one in either
   // kernel, and here both softmax warpgroups share its columns.  us a call, here / there: 2 heads x 4096 tokens, d = 64 30.7 /
   // 39.9, d = 128 35.9 / 44.1; 2 x 4500, d = 64 30.0 / 37.9.
-  if (p.block_k == 64 && (long long)p.call_heads * p.Nq > sms)
+  if (p.block_k == 64 && p.mode != SOL_MODE_DENSE && (long long)p.call_heads * p.Nq > sms)
     return fwd::launch_b64(p, q, k, v, out, ws, tau, counts, mask_out, fwd::g_wait_limit, fwd::g_withhold_tile, stream,
                            n_launches);
   fwd::Maps m;

@@ -135,8 +135,7 @@ __device__ void router_role(Shared<C>& sm, const Params& p, int lane) {
   const int n_chunks = ceil_div(p.Nk, kBlk);
   const int mask_words = ceil_div(p.Nk, 32);
   const float inv_sl2 = 1.f / (p.scale * 1.4426950408889634f);   // biases are stored in raw-score units
-  constexpr bool from_mask = kFromMask;
-  const bool score = p.mode != SOL_MODE_DENSE && !from_mask;
+  constexpr bool from_mask = kFromMask, score = !kFromMask;
   const float bias_full = log2f((float)kBlk) * inv_sl2;                          // log2 n_j of a full block ...
   const float bias_last = log2f((float)(p.N - (p.Nk - 1) * kBlk)) * inv_sl2;     // ... and of the ragged last one
   bool alive = true;
@@ -259,9 +258,7 @@ __device__ void router_role(Shared<C>& sm, const Params& p, int lane) {
         for (int u = 0; u < kNQ; ++u) {
           const bool exists = (valid >> u) & 1;
           bool sel;
-          if (p.mode == SOL_MODE_DENSE) {
-            sel = in_range;
-          } else if (from_mask) {
+          if (from_mask) {
             sel = exists && in_range &&
                   ((p.mask_out[(row0 + u / step) * mask_words + jbase / 32] >> lane) & 1u);
           } else {
@@ -858,8 +855,7 @@ fwd_sm100_b64_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
 template <class C>
 cudaError_t launch_instance(const Problem& p, const Maps& m, const Params& prm, int grid, cudaStream_t stream) {
   const size_t smem = 2 * C::kQBytes + 2 * kStages * C::kTileBytes + sizeof(Shared<C>);
-  auto kernel = p.routing == SOL_ROUTING_PREPASS && p.mode != SOL_MODE_DENSE ? fwd_sm100_b64_kernel<C, true>
-                                                                            : fwd_sm100_b64_kernel<C, false>;
+  auto kernel = p.routing == SOL_ROUTING_PREPASS ? fwd_sm100_b64_kernel<C, true> : fwd_sm100_b64_kernel<C, false>;
   return launch_after(kernel, dim3(grid), kThreads64, smem, smem, 0, stream, m.q, m.k, m.v, m.kc, m.vm, prm);
 }
 

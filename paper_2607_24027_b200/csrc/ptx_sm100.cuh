@@ -44,20 +44,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Has the phase completed?  Never suspends the thread (try_wait may, for as long as the hardware likes), so it
-// is the one to use where the caller has other work that the phase may depend on.
-__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_addr(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
 // Bounded wait on an mbarrier phase.  Gives up after ~`limit` SM clocks (kWaitCycles unless the
 // caller says otherwise) or as soon as another thread of the CTA has flagged an abort; returns
 // false in that case.
