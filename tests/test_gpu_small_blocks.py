@@ -127,3 +127,30 @@ def test_not_finite_inputs_with_several_blocks_per_item():
     err = (out[0].double() - ref[0]).abs()[good]
     assert bool((err <= torch.clamp(ref[0][good].abs() * 1e-2, min=hp.MAX_ABS)).all()), float(err.max())
     assert bool((out[0][~good] == 0).all())
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("routing", ["fused", "prepass"])
+def test_bounded_wait_runs_out(d, routing):
+    """A value tile's slot that is never handed back, in a ring of four, with 24 tiles per work item: the waits run out after
+    about a millisecond, every role drains what it has in flight, and the same workspace serves the next call."""
+    from paper_2607_24027_b200 import binding as sb
+    H, N = 40, 64 * 24
+    q, k, v = _many_blocks(1, H, N, d, 11)
+    route = sb.SOL_ROUTING_PREPASS if routing == "prepass" else sb.SOL_ROUTING_FUSED
+    good, counts, _, ws = hp.run_gpu(q, k, v, 64, -float("inf"), routing=route)
+    assert bool((counts == 24).all())
+    out, mask = torch.empty_like(q), torch.zeros(1, H, 24, 1, dtype=torch.int32, device="cuda")
+    sb.sol_attn_debug_set_wait(2_000_000, 1)
+    try:
+        sb.sol_attn_forward_ex(q, k, v, out, ws, 64, 64, threshold=-float("inf"), mask_out=mask, routing=route)
+        torch.cuda.synchronize()
+        detail = int(ws.buf[:8].view(torch.int32)[1].item())
+        sb.sol_attn_bind_workspace(ws)
+        st = sb.sol_attn_read_device_status()
+    finally:
+        sb.sol_attn_debug_set_wait(0, -1)
+    assert st == sb.SOL_ERR_DEVICE_TIMEOUT, sb.status_string(st)
+    assert detail != 0                                       # where the first wait gave up
+    again, counts, _, _ = hp.run_gpu(q, k, v, 64, -float("inf"), routing=route, ws=ws)
+    assert torch.equal(again, good) and bool((counts == 24).all())
