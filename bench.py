@@ -452,7 +452,7 @@ def main():
                    "topk_ms": ms_topk, "topp_ms": ms_topp,
                    "topk_over_thresholds": ms_topk / ms_thr, "topp_over_thresholds": ms_topp / ms_thr,
                    "materialised_bytes": int(pmap.numel() * 4 + order.numel() * 4),
-                   "note": "thresholds: mean, covariance and tau kernels on pooled data (nothing of size Nq x Nk "
+                   "note": "thresholds: one kernel on pooled data (nothing of size Nq x Nk "
                            "exists); mask_prepass: the optional SOL_ROUTING_PREPASS kernel, one bit per block pair; baselines: "
                            "proxy map + routing indices in HBM, k = %d blocks, p = 0.9" % k_blocks}
         check_status()

@@ -602,8 +602,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 fwd_sm100_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_kc,
                  const __grid_constant__ CUtensorMap tm_vm, const Params p) {
-  // (aligned by declaration and not by rounding the pointer, so that every address in it is a constant: 105.5 -> 103.5 us at
-  //  24 heads x 4096 tokens, d = 128; with both this and the waits out of line 103.4)
+  // (aligned by declaration and not by rounding the pointer, so that every address in it is a constant.  us, rounded / declared,
+  //  24 heads x 4096 tokens, d = 128: 99.2 / 97.9, and 100.8 / 98.9 where the waits spin inline (see ptx_sm100.cuh))
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* base = smem_raw;
   unsigned char* sQ = base;

@@ -569,8 +569,11 @@ __global__ void __launch_bounds__(256) tau_diag_kernel(WsPtrs ws, int Nq, float 
 // CTAs per head of thresholds_moments_kernel: the size with the least time.  `cycles` is a CTA's time in thousands (591 x 591
 // blocks, d = 128; other sizes are in much the same proportions).  As many CTAs as find an SM of their own run at that pace:
 // clusters of 1 and 2 fill the GPU, clusters of 3 to 6 about 17/20 of it, and of clusters of 8 no more than 14 are placed at
-// once.  Two CTAs on an SM share its FMA pipes and take 1.8 times as long.  us with the size taken / others: 40 heads x 591 blocks
-// (3) 58 / 6: 64, 2: 84; 16 x 591 (6) 41 / 8: 52; 48 x 300 (5) 35 / 2: 46; 80 x 300 (3) 57 / 1: 78.
+// once.  Two CTAs on an SM share its FMA pipes and take 1.8 times as long.  The table was taken before the quadratic form's loop was
+// unrolled, which made the larger clusters more alike (a CTA's time, us of a call: 8 31.6, 6 and 5 38, 4 45, 3 55, 2 78, 1 132); the
+// sizes taken are still the best of all at each of these: us with the size taken / others, d = 128: 40 heads x 591 blocks
+// (3) 55.7 / 5: 61, 6: 69, 4: 76, 2: 79; 16 x 591 (6) 38.8 / 4: 45, 8: 50; 28 x 591 (4) 45.6 / 8: 51, 3: 56; 48 x 300 (5) 36 / 2: 47;
+// 80 x 300 (3) 58 / 5: 60, 2: 74; 100 x 160 (2) 45.3 / 1: 47; d = 64: 40 x 591 (3) 25.9 / 5: 27.5; 24 x 591 (5) 19.9 / 4: 21.
 static int cluster_size(int heads, int sms) {
   struct { int n, cycles; } const sizes[] = {{8, 46}, {6, 53}, {5, 58}, {4, 82}, {3, 95}, {2, 141}, {1, 268}};
   int best = 1;

@@ -50,8 +50,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 //
 // Only the first look is inline.  The fused kernels have four to six roles with code of their own in 45 to 65 KB, more than an SM's
 // instruction caches hold beside the unrolled softmax loop, and a role that runs a few hundred instructions once per
-// tile finds them evicted: the less of it, the sooner a role is through (us, spinning inline / out of line: 24 heads x 4096 tokens
-// 105.5 / 103.5, with 77 text tokens as a batch of two 242 / 239, 64-token blocks 16 x 11 160 d = 64 318 / 312).
+// tile finds them evicted: the less of it, the sooner a role is through.  us, spinning inline / out of line, 24 heads x 4096 tokens:
+// 98.9 / 97.9, and 100.8 / 99.2 where shared memory is aligned by rounding a pointer (see fwd_sm100.cu); 40 x 32 760 5570 / 5490.
 constexpr long long kWaitCycles = 4000000000LL;   // about 2-3 s of SM clocks
 static __device__ __noinline__ bool mbar_keep_waiting(uint64_t* bar, uint32_t parity, volatile int* abort_flag, long long limit) {
   const long long t0 = clock64();
